@@ -1337,7 +1337,7 @@ static clv_status mlp_grad_attr() {
 
 // blocks of a deterministic gradient launch over `batch` samples
 static int mlp_grad_blocks(long long batch) {
-  return (int)std::min<long long>(kMlpGradBlocks, (batch + kMlpTrainBlock - 1) / kMlpTrainBlock);
+  return (int)std::min<long long>(kMlpGradBlocks, (batch + kMlpChunk - 1) / kMlpChunk);
 }
 
 clv_status clv_mlp_loss_grad(const float* d_params, const float* d_X, const float* d_Y, int64_t n, void* stream,
@@ -1348,8 +1348,9 @@ clv_status clv_mlp_loss_grad(const float* d_params, const float* d_X, const floa
   if (s != CLV_OK) return s;
   cudaStream_t st = (cudaStream_t)stream;
   const int blocks = mlp_grad_blocks(n);
-  mlp_grad_kernel<<<blocks, kMlpTrainBlock, mlp_grad_smem_bytes(), st>>>(d_params, d_X, d_Y, n, n, 0ull, 0, d_work);
-  mlp_reduce_kernel<<<(kMlpPartialRow + 255) / 256, 256, 0, st>>>(d_work, blocks, d_grad, d_loss);
+  mlp_grad_kernel<<<blocks, kMlpGradThreads, mlp_grad_smem_bytes(), st>>>(d_params, d_X, d_Y, n, n, 0ull, 0, d_work);
+  mlp_reduce_kernel<<<(kMlpPartialRow + 31) / 32, 32 * kMlpReduceGroups, 0, st>>>(d_work, blocks, d_grad, d_loss,
+                                                                                  MlpAdam{});
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? CLV_OK : fail(nullptr, CLV_ECUDA, cudaGetErrorString(e));
 }
@@ -1367,10 +1368,10 @@ clv_status clv_mlp_train(float* d_params, float* d_work, const float* d_X, const
   float* partial = d_work + 3 * kMlpParams;
   const int blocks = mlp_grad_blocks(batch);
   for (int it = 0; it < iters; ++it) {
-    mlp_grad_kernel<<<blocks, kMlpTrainBlock, mlp_grad_smem_bytes(), st>>>(d_params, d_X, d_Y, n, batch, seed,
-                                                                          step0 + it, partial);
-    mlp_reduce_kernel<<<(kMlpPartialRow + 255) / 256, 256, 0, st>>>(partial, blocks, g, d_loss + it);
-    mlp_adam_kernel<<<(kMlpParams + 255) / 256, 256, 0, st>>>(d_params, m, v, g, step0 + it + 1, lr);
+    mlp_grad_kernel<<<blocks, kMlpGradThreads, mlp_grad_smem_bytes(), st>>>(d_params, d_X, d_Y, n, batch, seed,
+                                                                           step0 + it, partial);
+    mlp_reduce_kernel<<<(kMlpPartialRow + 31) / 32, 32 * kMlpReduceGroups, 0, st>>>(
+        partial, blocks, g, d_loss + it, MlpAdam{d_params, m, v, step0 + it + 1, lr});
   }
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? CLV_OK : fail(nullptr, CLV_ECUDA, cudaGetErrorString(e));
