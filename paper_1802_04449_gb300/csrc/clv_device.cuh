@@ -93,8 +93,11 @@ __device__ __forceinline__ void eos_eval(const EosView<R>& q, C e, C& P, C& T, C
     // relative noise from the lookup alone.  So x is never formed as one
     // float: x = xk[ex] + ln(m)/dlne with ln(m) in (-0.7, 0] to ~1e-7, and the
     // fraction of the sum is exact to ~1e-5 of a node interval.
-    int ex;
-    const float m = frexpf(e, &ex);
+    // frexp of a positive float by its bits (a subnormal's exponent field
+    // gives ex = -126: below the table, as its true exponent would)
+    const unsigned bits = __float_as_uint(e);
+    const int ex = (int)(bits >> 23) - 126;
+    const float m = __uint_as_float((bits & 0x007fffffu) | 0x3f000000u);
     if (ex < -125) {
       k = -1;
       w = C(0);

@@ -109,6 +109,11 @@ template <typename R> __device__ __forceinline__ R ldg(const R* p) { return __ld
 template <typename R> struct SolveTraits;
 template <> struct SolveTraits<float> {
   static constexpr float tol = 5e-7f;
+  // last step of a solve that a further Newton step follows: below v = 0.99
+  // the step's error is 0.5 |dv|^2 or less plus |dv| times the mismatch of
+  // the tabulated c_s^2 and the table's slope (1e-3): 2e-8 at 2e-5, under the
+  // 1e-7 of the FP32 residual that ends either solve
+  static constexpr float tol_corrected = 2e-5f;
   static constexpr int maxit = 40;
 };
 template <> struct SolveTraits<double> {
@@ -760,8 +765,15 @@ __global__ void __launch_bounds__(kBlock, RecoverMinBlocks<R>::value) recover_ke
     if (!(isfinite(E) && isfinite(Mx) && isfinite(My) && isfinite(Me))) {
       f_nonfinite = true;
     } else {
-      RootResult rr = solve_primitive<R, R>(p.eos, p.eps_cut, E, Mx, My, Me, SolveTraits<R>::tol,
-                                            SolveTraits<R>::maxit, en, ux, uy, ue, &vg, &at_root, Pb);
+      // FP32: a cell below the velocity threshold of the FP64 refinement gets
+      // a Newton step of its own below (correct_root, or the refinement near
+      // the cut), which takes a root known to tol_corrected to the same
+      // result as one known to tol
+      R tol = SolveTraits<R>::tol;
+      if constexpr (sizeof(R) == 4)
+        if (Mx * Mx + My * My + Me * Me <= (p.polish_v * E) * (p.polish_v * E)) tol = SolveTraits<R>::tol_corrected;
+      RootResult rr = solve_primitive<R, R>(p.eos, p.eps_cut, E, Mx, My, Me, tol, SolveTraits<R>::maxit, en, ux, uy,
+                                            ue, &vg, &at_root, Pb);
       f_rescaled = rr.rescaled;
       my_iters = rr.iters > 0 ? rr.iters : 0;
       my_solved = rr.iters > 0 ? 1 : 0;
