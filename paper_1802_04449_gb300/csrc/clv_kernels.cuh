@@ -154,7 +154,11 @@ __device__ __forceinline__ void interface_flux(const R* L, const R* Rr, R csl, R
   constexpr int IU = VISC ? 14 : 4, IV = IU + 1, IP = IU + 2;
   const R vl = L[IV], vr = Rr[IV];
   const R al = fabs(vl), ar = fabs(vr);
-  const R lam = fmax((al + csl) / (R(1) + al * csl), (ar + csr) / (R(1) + ar * csr));
+  // lam = max of (|v| + c_s)/(1 + |v| c_s) of the two sides, the larger one
+  // found by cross-multiplication: one division
+  const R nl = al + csl, dl = R(1) + al * csl, nr = ar + csr, dr = R(1) + ar * csr;
+  const bool rs = nr * dl > nl * dr;
+  const R lam = (rs ? nr : nl) / (rs ? dr : dl);
   // H = (F_l + F_r)/2 - lam (Q_r - Q_l)/2 with F = v Q + tau X regrouped as
   // wl Q_l + wr Q_r + tau (X_l + X_r)/2, wl = (v_l + lam)/2, wr = (v_r - lam)/2
   const R wl = R(0.5) * (vl + lam), wr = R(0.5) * (vr - lam);
@@ -162,14 +166,18 @@ __device__ __forceinline__ void interface_flux(const R* L, const R* Rr, R csl, R
 #pragma unroll
   for (int m = 0; m < 4; ++m) {
     // X of T~^{tau m} along a: P (v d_{m tau} + d_{m a}) + pi~^{a m} - v pi~^{tau m}
-    R gl = (m == 0 ? vl : R(0)) + (m == axis ? R(1) : R(0));
-    R gr = (m == 0 ? vr : R(0)) + (m == axis ? R(1) : R(0));
-    R xl = L[IP] * gl, xr = Rr[IP] * gr;
+    R h = wl * L[m] + wr * Rr[m];
     if constexpr (VISC) {
-      xl += L[4 + sym_index(axis, m)] - vl * L[4 + sym_index(0, m)];
-      xr += Rr[4 + sym_index(axis, m)] - vr * Rr[4 + sym_index(0, m)];
+      R xl = L[4 + sym_index(axis, m)] - vl * L[4 + sym_index(0, m)];
+      R xr = Rr[4 + sym_index(axis, m)] - vr * Rr[4 + sym_index(0, m)];
+      if (m == 0) { xl += vl * L[IP]; xr += vr * Rr[IP]; }
+      if (m == axis) { xl += L[IP]; xr += Rr[IP]; }
+      h += ht * (xl + xr);
+    } else {
+      if (m == 0) h += ht * (vl * L[IP] + vr * Rr[IP]);
+      if (m == axis) h += ht * (L[IP] + Rr[IP]);
     }
-    H[m] = wl * L[m] + wr * Rr[m] + ht * (xl + xr);
+    H[m] = h;
   }
   if constexpr (VISC) {
     // Q_pi = u~^tau pi~ on each side, flux v Q_pi
@@ -333,15 +341,22 @@ __device__ __forceinline__ void shear_source(R geo, const R u[4], R du[4][4], co
            pi[sym_index(m, 3)] * Du[3];
   const R ep5 = (e + P) * is.inv_b;
   const R decay = inv_taupi + theta * R(1.0 / 3.0) + geo * u[0];
+  // ep5 sigma^{mn} - (u^m w^n + u^n w^m) with sigma^{mn} = g^m d_m u^n + g^n
+  // d_n u^m - u^m Du^n - u^n Du^m - (2/3) (g^{mn} - u^m u^n) theta, gathered
+  // as ep5 (...) + u^m C^n + u^n C^m, C^m = ep5 (theta u^m / 3 - Du^m) - w^m
+  const R th23 = R(2.0 / 3.0) * theta;
+  R C[4];
+#pragma unroll
+  for (int m = 0; m < 4; ++m) C[m] = ep5 * (R(0.5) * th23 * u[m] - Du[m]) - w[m];
 #pragma unroll
   for (int m = 0; m < 4; ++m)
 #pragma unroll
     for (int n = m; n < 4; ++n) {
       const int q = sym_index(m, n);
       const R sm = R(metric_sign(m)), sn = R(metric_sign(n));
-      R sigma = sm * du[m][n] + sn * du[n][m] - u[m] * Du[n] - u[n] * Du[m] -
-                R(2.0 / 3.0) * ((m == n ? sm : R(0)) - u[m] * u[n]) * theta;
-      S[q] = ep5 * sigma - decay * pi[q] - (u[m] * w[n] + u[n] * w[m]);
+      R d = sm * du[m][n] + sn * du[n][m];
+      if (m == n) d -= sm * th23;
+      S[q] = ep5 * d + u[m] * C[n] + u[n] * C[m] - decay * pi[q];
     }
   // -(lambda_1 / tau_pi) pi^<mu_l pi^nu>l in tilde components: Y = pi g~ pi,
   // X = Delta^m_a Delta^n_c Y^ac - Delta^mn (Delta_ac Y^ac) / 3
@@ -449,7 +464,7 @@ __global__ void __launch_bounds__(kBlock) stage_kernel(const StageParams<R> p) {
           else if (q == IV) v[d] = va[d];
           else v[d] = ldg(p.pr.P + id[d]);
         }
-        const R s1 = minmod(v[1] - v[0], v[2] - v[1]);
+        const R s1 = minmod(v[2] - v[1], v[1] - v[0]);
         const R s2 = minmod(v[2] - v[1], v[3] - v[2]);
         const R s3 = minmod(v[3] - v[2], v[4] - v[3]);
         Lm[q] = v[1] + R(0.5) * s1;
@@ -540,9 +555,9 @@ __global__ void __launch_bounds__(kBlock) stage_kernel(const StageParams<R> p) {
         }
       }
       if constexpr (VISC) {
-        const R inv = R(1) / ustar0;
+        const R inv = R(1) / ustar0, cn = un[0] * inv, ch = h * inv;
 #pragma unroll
-        for (int q = 0; q < 10; ++q) pinew[q] = (un[0] * pic[q] + h * S[4 + q]) * inv;
+        for (int q = 0; q < 10; ++q) pinew[q] = cn * pic[q] + ch * S[4 + q];
         regulate_shear<R>(e, Pe, pinew);
       }
     } else {
@@ -557,9 +572,9 @@ __global__ void __launch_bounds__(kBlock) stage_kernel(const StageParams<R> p) {
         }
       }
       if constexpr (VISC) {
-        const R inv = R(0.5) / u[0];
+        const R inv = R(0.5) / u[0], cn = un[0] * inv, cs = ustar0 * inv, ch = h * inv;
 #pragma unroll
-        for (int q = 0; q < 10; ++q) pinew[q] = (un[0] * p.pin[q][c] + ustar0 * pic[q] + h * S[4 + q]) * inv;
+        for (int q = 0; q < 10; ++q) pinew[q] = cn * p.pin[q][c] + cs * pic[q] + ch * S[4 + q];
         regulate_shear<R>(e, Pe, pinew);
       }
     }

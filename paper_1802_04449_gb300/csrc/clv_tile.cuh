@@ -190,7 +190,7 @@ __device__ __forceinline__ void box_interface(const R* box, int NB, int c, int s
     const int f = q < L::UT ? q : (q == L::UT ? L::UT : (q == L::UT + 1 ? L::V + ax - 1 : L::P));
     const R* col = box + f * NB + c;
     const R v0 = col[-2 * stride], v1 = col[-stride], v2 = col[0], v3 = col[stride];
-    Ls[q] = v1 + R(0.5) * minmod(v1 - v0, v2 - v1);
+    Ls[q] = v1 + R(0.5) * minmod(v2 - v1, v1 - v0);
     Rs[q] = v2 - R(0.5) * minmod(v2 - v1, v3 - v2);
   }
   const R* cs = box + L::CS * NB + c;
@@ -440,9 +440,9 @@ __device__ __forceinline__ void stage_tile_body(const StageParams<R>& p, const E
                 }
               }
               if constexpr (VISC) {
-                const R inv = R(1) / ustar0;
+                const R inv = R(1) / ustar0, cn = un[0] * inv, ch = hh * inv;
 #pragma unroll
-                for (int r = 0; r < 10; ++r) pinew[r] = (un[0] * W0[4 + r] + hh * S[4 + r]) * inv;
+                for (int r = 0; r < 10; ++r) pinew[r] = cn * W0[4 + r] + ch * S[4 + r];
                 regulate_shear<R>(e, Pe, pinew);
               }
             } else {
@@ -459,10 +459,10 @@ __device__ __forceinline__ void stage_tile_body(const StageParams<R>& p, const E
                 }
               }
               if constexpr (VISC) {
-                const R inv = R(0.5) / u[0];
+                const R inv = R(0.5) / u[0], cn = un[0] * inv, cs = ustar0 * inv, ch = hh * inv;
 #pragma unroll
                 for (int r = 0; r < 10; ++r)
-                  pinew[r] = (un[0] * cb[(CI::PIN + r) * ncell] + ustar0 * W0[4 + r] + hh * S[4 + r]) * inv;
+                  pinew[r] = cn * cb[(CI::PIN + r) * ncell] + cs * W0[4 + r] + ch * S[4 + r];
                 regulate_shear<R>(e, Pe, pinew);
               }
             }
