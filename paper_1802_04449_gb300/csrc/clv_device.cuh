@@ -373,6 +373,14 @@ __device__ __forceinline__ void cp_async_wait_prior() { asm volatile("cp.async.w
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 
+// sqrt(a) and 1/sqrt(a), a >= 1, from one reciprocal square root and a
+// correction of the root (its residual a - r^2 is exact by FMA)
+__device__ __forceinline__ void sqrt_and_inverse(double a, double& root, double& inv) {
+  inv = rsqrt(a);
+  const double r = mul_rn(a, inv);
+  root = fma(fma(-r, r, a), 0.5 * inv, r);
+}
+
 // minmod(a, b): 0 unless a and b share a sign, else the one of smaller
 // magnitude (the value is a, b or 0 exactly).  FP32: b clamped to the
 // interval between 0 and a, four min/max operations on the ALU pipe.  FP64:

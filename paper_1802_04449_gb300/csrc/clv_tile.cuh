@@ -106,12 +106,19 @@ __device__ __forceinline__ void cp_async_vec4(double* smem, const double* gmem) 
 // in-plane offset of a vector inside the grid's eta range (.y < 0: one
 // vector copy) or the four offsets, clamped or wrapped at the boundary, of a
 // vector that crosses it.  Thread tid handles vectors w = tid, tid + nthr,
-// ... < nvec; the caller commits the group.
+// ... < nvec; FP64: bits 4 r .. 4 r + 3 of mask (r = 0, 1, ...) say which of
+// their cells the plane needs, and a vector with none is left out.  The caller
+// commits the group.
 template <typename R, bool VISC>
 __device__ __forceinline__ void stage_plane_async(const StageParams<R>& p, R* box, int nvec, long long poff,
-                                                  const int4* voff, int tid, int nthr, int NB) {
+                                                  const int4* voff, unsigned mask, int tid, int nthr, int NB) {
   using L = Box<VISC>;
   for (int w = tid; w < nvec; w += nthr) {
+    if constexpr (sizeof(R) == 8) {
+      const bool none = !(mask & 15u);
+      mask >>= 4;
+      if (none) continue;
+    }
     const int4 o = voff[w];
     R* d = box + 4 * w;
     auto copy = [&](R* dst, const R* src) {
@@ -271,8 +278,23 @@ __device__ __forceinline__ void stage_tile_body(const StageParams<R>& p, const E
 
   // in-plane offsets of this thread's box vectors (only this thread uses them)
   const int vend = worker ? NV : 0;   // vectors this thread stages: w = tid, tid + nthr, ... < vend
-  for (int w = tid; w < vend; w += nthr) {
+  // FP64 also: the cells of them that a plane needs -- an output plane the
+  // tile with its halo (no corners), the two planes on either side of the
+  // chunk only the tile's own columns (their x-stencil).  The conversion to v
+  // costs a square root and a division of a cell on the narrow FP64 pipe, and
+  // with few planes to a chunk most of the box is not needed: the stage of a
+  // 33 x 33 x 9 ideal event 38.7 -> 35.6 us; FP32 converts whole vectors (the
+  // tests cost it what they save).  A thread has at most 4 vectors: (TJ + 4)
+  // box_width(TK) / 4 <= 3.5 (TJ + 1) (TK + 1).
+  unsigned need_out = 0, need_own = 0;
+  for (int w = tid, sh = 0; w < vend; w += nthr, sh += 4) {
     const int bj = (4 * w) / BW, c0 = kb0 + 4 * w - bj * BW;
+    for (int i = 0; i < 4 && sizeof(R) == 8; ++i) {
+      const int col = c0 + i - k0;
+      const bool in_j = bj >= 2 && bj < t.TJ + 2, in_k = col >= 0 && col < t.TK;
+      need_own |= (in_j && in_k ? 1u : 0u) << (sh + i);
+      need_out |= (in_k || (in_j && col >= -2 && col < t.TK + 2) ? 1u : 0u) << (sh + i);
+    }
     const int row = wrap_index(j0 + bj - 2, ev.ny, p.periodic) * ev.nep;
     if (c0 >= 0 && c0 + 3 < ev.ne)
       voff[w] = make_int4(row + c0, -1, 0, 0);
@@ -286,8 +308,8 @@ __device__ __forceinline__ void stage_tile_body(const StageParams<R>& p, const E
   // Copy groups of a thread alternate: a plane group, then a cell group
   // (the per-cell inputs of its next output cell), each possibly empty, so
   // that waiting for all but the newest group lands exactly the one needed.
-  stage_plane_async<R, VISC>(p, boxbuf + ((x0 - 2) & 1) * NF * NB, vend, ev.off + xplane(x0 - 2) * plane, voff, tid,
-                             nthr, NB);
+  stage_plane_async<R, VISC>(p, boxbuf + ((x0 - 2) & 1) * NF * NB, vend, ev.off + xplane(x0 - 2) * plane, voff,
+                             need_own, tid, nthr, NB);
   cp_async_commit();
   cp_async_commit();   // no cell group before the first plane
   for (int pl = x0 - 2; pl <= x1 + 1; ++pl) {
@@ -297,13 +319,25 @@ __device__ __forceinline__ void stage_tile_body(const StageParams<R>& p, const E
     // committed after them may still be in flight): its u~ -> (u~^tau, v) in
     // place, then one barrier makes the whole plane visible
     cp_async_wait_prior();
+    unsigned mask = out_plane ? need_out : need_own;
     for (int w = tid; w < vend; w += nthr) {   // the cells of its vectors
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
+        if constexpr (sizeof(R) == 8) {
+          const bool skip = !(mask & 1u);
+          mask >>= 1;
+          if (skip) continue;
+        }
         const int q = 4 * w + i;
         const R ux = box[L::V * NB + q], uy = box[(L::V + 1) * NB + q], ue = box[(L::V + 2) * NB + q];
-        const R ut = sqrt(R(1) + ux * ux + uy * uy + ue * ue);
-        const R iu = R(1) / ut;
+        const R a = R(1) + ux * ux + uy * uy + ue * ue;
+        R ut, iu;
+        if constexpr (sizeof(R) == 8) {
+          sqrt_and_inverse(a, ut, iu);
+        } else {
+          ut = sqrt(a);
+          iu = R(1) / ut;
+        }
         box[L::UT * NB + q] = ut;
         box[L::V * NB + q] = ux * iu;
         box[(L::V + 1) * NB + q] = uy * iu;
@@ -314,7 +348,8 @@ __device__ __forceinline__ void stage_tile_body(const StageParams<R>& p, const E
     // prefetch the next plane into the other buffer while this one is used
     if (pl + 1 <= x1 + 1)
       stage_plane_async<R, VISC>(p, boxbuf + ((pl + 1) & 1) * NF * NB, vend,
-                                 ev.off + xplane(pl + 1) * plane, voff, tid, nthr, NB);
+                                 ev.off + xplane(pl + 1) * plane, voff,
+                                 pl + 1 >= x0 && pl + 1 < x1 ? need_out : need_own, tid, nthr, NB);
     cp_async_commit();
     // ---- 2. every y- and eta-interface of an output plane, once
     if (out_plane) {
