@@ -70,10 +70,19 @@ __device__ __forceinline__ Node<double> load_node(const double* base, int k) {
   return {a.x, a.y, b.x, 0.0};
 }
 
+// The interpolant around a looked-up e: dP/de = num/den and d(c_s^2)/de =
+// dc2/den there, and the part (0 .. 1/2) of a node interval in ln e that can
+// be moved either way inside the same piece (0: do not).
+template <typename C> struct EosLocal {
+  C num, den, dc2, room;
+};
+
 // Evaluate in arithmetic type C (C may be wider than the table type R).
 template <typename C, typename R>
-__device__ __forceinline__ void eos_eval(const EosView<R>& q, C e, C& P, C& T, C& cs2) {
+__device__ __forceinline__ void eos_eval(const EosView<R>& q, C e, C& P, C& T, C& cs2, EosLocal<C>* loc = nullptr) {
+  if (loc) *loc = EosLocal<C>{C(1.0 / 3.0), C(1), C(0), C(0)};
   if (q.kind == 0) {
+    if (loc) loc->room = C(0.5);
     P = e * C(1.0 / 3.0);
     cs2 = C(1.0 / 3.0);
     T = (e > C(0)) ? sqrt(sqrt(C(q.t_coef) * e)) : C(0);
@@ -83,6 +92,7 @@ __device__ __forceinline__ void eos_eval(const EosView<R>& q, C e, C& P, C& T, C
     P = C(0);
     T = C(0);
     cs2 = C(load_node(q.node, 0).c2);
+    if (loc) loc->num = cs2;
     return;
   }
   int k;
@@ -122,6 +132,7 @@ __device__ __forceinline__ void eos_eval(const EosView<R>& q, C e, C& P, C& T, C
     P = C(a.P) * r;
     T = C(a.T) * sqrt(sqrt(r));
     cs2 = C(a.c2);
+    if (loc) { loc->num = C(a.P); loc->den = C(q.e0); }
     return;
   }
   if (k >= q.n - 1) {
@@ -136,6 +147,12 @@ __device__ __forceinline__ void eos_eval(const EosView<R>& q, C e, C& P, C& T, C
   if constexpr (sizeof(R) == 4) P += C(a.Plo) + w * (C(b.Plo) - C(a.Plo));
   T = C(a.T) + w * (C(b.T) - C(a.T));
   cs2 = C(a.c2) + w * (C(b.c2) - C(a.c2));
+  if (loc) {
+    loc->num = (C(b.P) - C(a.P)) * C(q.inv_dlne);
+    loc->den = e;
+    loc->dc2 = (C(b.c2) - C(a.c2)) * C(q.inv_dlne);
+    loc->room = w < C(0.5) ? w : C(1) - w;
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -252,16 +269,36 @@ __device__ __forceinline__ RootResult solve_primitive(const EosView<R>& q, C eps
   int it = 1;
   bool ok = false;
   C e_last = C(0);
+  EosLocal<CE> loc;
   for (; it <= maxit; ++it) {
     C e = E - M * v;
     e_last = e;
     {
       CE Pe, Te, ce;
-      eos_eval<CE, R>(q, CE(e), Pe, Te, ce);
+      eos_eval<CE, R>(q, CE(e), Pe, Te, ce, sizeof(CE) == 8 ? &loc : nullptr);
       P = C(Pe) + Pshift;
       cs2 = C(ce);
       dPde = cs2;
-      if (P < C(0)) { P = C(0); dPde = C(0); }
+      if (P < C(0)) { P = C(0); dPde = C(0); loc.num = CE(0); loc.room = CE(0); }
+    }
+    if constexpr (sizeof(CE) == 8) {
+      // FP64 lookups: the slope num/den of the interpolant itself (the
+      // tabulated c_s^2 differs from it by ~1e-3, which would leave the steps
+      // converging linearly at that rate), with the division folded into the
+      // step's
+      const C den = E + P, g = v * den - M;
+      if (g > C(0)) hi = v; else lo = v;
+      const C dv = -Ops::div(den * g * loc.den, den * den * loc.den - loc.num * (M * M));
+      // converged when the step is below tol, or when it moves eps by less
+      // than 1e-8 of itself within one piece of the interpolant: the step's
+      // error is then of second order, below 1e-16
+      const C de = fabs(M * dv);
+      if (fabs(dv) <= tol || (de <= C(1e-8) * e && de * C(q.inv_dlne) < loc.room * e)) { v += dv; ok = true; break; }
+      C vn = v + dv;
+      if (!(vn > lo && vn < hi)) vn = C(0.5) * (lo + hi);
+      v = vn;
+      if (hi - lo <= tol) { ok = true; break; }
+      continue;
     }
     // Newton step on f(v) = v - M/den, den = E + P: with g = v den - M
     // (the sign of f, den > 0) the step -f/f' is -den g / (den^2 - c_s^2 M^2),
@@ -269,7 +306,11 @@ __device__ __forceinline__ RootResult solve_primitive(const EosView<R>& q, C eps
     const C den = E + P;
     const C g = v * den - M;
     if (g > C(0)) hi = v; else lo = v;
-    const C dv = -Ops::div(den * g, den * den - dPde * (M * M));
+    C dv = -Ops::div(den * g, den * den - dPde * (M * M));
+    // an FP32 lookup no longer sees a step of eps below its rounding: P is
+    // constant there, and the step that takes it so lands on the root
+    if constexpr (sizeof(CE) < sizeof(C))
+      if (fabs(M * dv) <= C(6e-8) * e) dv = -Ops::div(g, den);
     // converged when the Newton step is below tol; otherwise keep the iterate
     // strictly inside the shrinking bracket
     if (fabs(dv) <= tol) { v += dv; ok = true; break; }
@@ -286,8 +327,14 @@ __device__ __forceinline__ RootResult solve_primitive(const EosView<R>& q, C eps
   eps = e;
   if (at_root) {
     at_root->valid = true;
-    at_root->P = P + dPde * (e - e_last);
-    at_root->cs2 = cs2;
+    if constexpr (sizeof(CE) == 8) {
+      const C x = Ops::div(e - e_last, loc.den);
+      at_root->P = P + loc.num * x;
+      at_root->cs2 = cs2 + loc.dc2 * x;
+    } else {
+      at_root->P = P + dPde * (e - e_last);
+      at_root->cs2 = cs2;
+    }
   }
   C gam = Ops::rsqrt_(C(1) - v * v);
   C s = Ops::div(gam * v, M);
