@@ -92,8 +92,7 @@ struct clv_handle {
   double* block_sum = nullptr;    // nblocks doubles
   DevStats* dstats = nullptr;
   int sms = 148;                  // multiprocessors of the device
-  double* tau_dev = nullptr;      // tau of the step on the device (the kernels read it)
-  float* itau_dev = nullptr;      // 1/tau at the end of the step as a float-float pair (FP32 recovery)
+  TauSlot* tau_dev = nullptr;     // [2] tau on the device (the kernels read it), slot cur for the next step
   double tau = 0.0;               // host copy, advanced by the same additions
   long long step = 0;
   bool initialized = false;
@@ -361,7 +360,7 @@ size_t layout(const clv_config* c, clv_handle* h) {
   size_t oStage = take(std::max((size_t)N * 8, (size_t)256));  // also scratch of clv_mlp_samples
   size_t oBlock = take((size_t)nblocks * 8);
   size_t oStats = take(sizeof(DevStats));
-  size_t oTau = take(4 * sizeof(double));   // tau (double), then 1/tau as two floats
+  size_t oTau = take(2 * sizeof(TauSlot));
   if (h) {
     char* b = h->ws;
     for (int m = 0; m < 4; ++m) { h->T0[m] = b + oT0[m] + hoff; h->T1[m] = b + oT1[m] + hoff; }
@@ -379,8 +378,7 @@ size_t layout(const clv_config* c, clv_handle* h) {
     h->staging = (double*)(b + oStage);
     h->block_sum = (double*)(b + oBlock);
     h->dstats = (DevStats*)(b + oStats);
-    h->tau_dev = (double*)(b + oTau);
-    h->itau_dev = (float*)(b + oTau + 2 * sizeof(double));
+    h->tau_dev = (TauSlot*)(b + oTau);
     h->nblocks = nblocks;
     h->N = N;
     h->Nc = (long long)c->nx * c->ny * c->neta;
@@ -458,8 +456,9 @@ StageParams<R> stage_params(clv_handle* h, int stage) {
   p.nep = h->nep;
   p.xhalo = c.halo_x > 0 ? 1 : 0;
   p.N = h->N;
-  p.tau_dev = h->tau_dev;
-  p.itau = h->itau_dev;
+  p.tau_dev = &h->tau_dev[h->cur].tau;
+  p.itau = h->tau_dev[h->cur].itau;
+  p.tau_next = s1 ? nullptr : h->tau_dev + h->prev;   // prev becomes cur after the step
   p.dtau_d = c.dtau;
   p.cartesian = c.cartesian;
   p.h = (R)c.dtau;
@@ -523,11 +522,11 @@ template <typename R, bool VISC> cudaError_t tile_attributes(size_t smem) {
 template <typename R, bool VISC, bool STATS> void launch_recover(clv_handle* h, const StageParams<R>& p) {
   const unsigned g = grid_of(h->N);
   if (sizeof(R) == 4 && h->guess == kGuessMlp)
-    recover_kernel<R, VISC, STATS, sizeof(R) == 4 ? kGuessMlp : kGuessPrevious><<<g, kBlock, 0, h->stream>>>(p);
+    launch_step_kernel(recover_kernel<R, VISC, STATS, sizeof(R) == 4 ? kGuessMlp : kGuessPrevious>, g, kBlock, 0, h->stream, p);
   else if (sizeof(R) == 4 && h->guess == kGuessMlpAll)
-    recover_kernel<R, VISC, STATS, sizeof(R) == 4 ? kGuessMlpAll : kGuessPrevious><<<g, kBlock, 0, h->stream>>>(p);
-  else if (h->guess == kGuessCold) recover_kernel<R, VISC, STATS, kGuessCold><<<g, kBlock, 0, h->stream>>>(p);
-  else recover_kernel<R, VISC, STATS, kGuessPrevious><<<g, kBlock, 0, h->stream>>>(p);
+    launch_step_kernel(recover_kernel<R, VISC, STATS, sizeof(R) == 4 ? kGuessMlpAll : kGuessPrevious>, g, kBlock, 0, h->stream, p);
+  else if (h->guess == kGuessCold) launch_step_kernel(recover_kernel<R, VISC, STATS, kGuessCold>, g, kBlock, 0, h->stream, p);
+  else launch_step_kernel(recover_kernel<R, VISC, STATS, kGuessPrevious>, g, kBlock, 0, h->stream, p);
 }
 
 // One stage: the stage kernel, then the root solve (the direct kernel does
@@ -536,47 +535,35 @@ template <typename R, bool VISC, int STAGE, bool STATS>
 void launch_stage(clv_handle* h, const StageParams<R>& p, bool timed) {
   if (!h->batch.empty()) {
     cudaMemsetAsync(h->batch_ctr + (STAGE - 1), 0, sizeof(int), h->stream);
-    stage_batch_kernel<R, STAGE, VISC><<<h->batch_blocks, h->batch_threads, h->batch_smem, h->stream>>>(
-        p, (const EventGeom<R>*)h->batch_geom, h->batch_tiles, h->batch_items, h->batch_nitems,
-        h->batch_ctr + (STAGE - 1));
+    launch_step_kernel(stage_batch_kernel<R, STAGE, VISC>, h->batch_blocks, h->batch_threads, h->batch_smem, h->stream,
+                       p, (const EventGeom<R>*)h->batch_geom, h->batch_tiles, h->batch_items, h->batch_nitems,
+                       h->batch_ctr + (STAGE - 1));
     if (timed) timing_event(h);
     launch_recover<R, VISC, STATS>(h, p);
   } else if (h->cfg.kernel == 1) {
-    stage_kernel<R, STAGE, VISC, STATS><<<grid_of(h->N), kBlock, 0, h->stream>>>(p);
+    launch_step_kernel(stage_kernel<R, STAGE, VISC, STATS>, grid_of(h->N), kBlock, 0, h->stream, p);
     if (timed) timing_event(h);   // empty recovery slot
   } else {
-    stage_tile_kernel<R, STAGE, VISC><<<h->tile_blocks, h->tile_threads, h->tile_smem, h->stream>>>(p, h->tile);
+    launch_step_kernel(stage_tile_kernel<R, STAGE, VISC>, h->tile_blocks, h->tile_threads, h->tile_smem, h->stream, p,
+                       h->tile);
     if (timed) timing_event(h);
     launch_recover<R, VISC, STATS>(h, p);
   }
   if (timed) timing_event(h);
 }
 
-// tau of the step, and 1/tau of the end of the step (tau + dtau; 1 in
-// Cartesian mode) as a float-float pair for the FP32 recovery
-__device__ __forceinline__ void store_itau(float* itau, double tau, double dtau, int cartesian) {
-  const double x = cartesian ? 1.0 : 1.0 / (tau + dtau);
-  const float hi = (float)x;
-  itau[0] = hi;
-  itau[1] = (float)(x - (double)hi);
-}
-__global__ void set_tau_kernel(double* tau_dev, float* itau, double tau, double dtau, int cartesian) {
-  *tau_dev = tau;
-  store_itau(itau, tau, dtau, cartesian);
-}
-__global__ void advance_tau_kernel(double* tau_dev, float* itau, double dtau, int cartesian) {
-  const double t = *tau_dev + dtau;
-  *tau_dev = t;
-  store_itau(itau, t, dtau, cartesian);
+__global__ void set_tau_kernel(TauSlot* s, double tau, double dtau, int cartesian) {
+  store_tau(s, tau, dtau, cartesian);
 }
 
+// tau of the next step (from the primitive set cur)
 void set_tau(clv_handle* h, double tau) {
   h->tau = tau;
-  set_tau_kernel<<<1, 1, 0, h->stream>>>(h->tau_dev, h->itau_dev, tau, h->cfg.dtau, h->cfg.cartesian);
+  set_tau_kernel<<<1, 1, 0, h->stream>>>(h->tau_dev + h->cur, tau, h->cfg.dtau, h->cfg.cartesian);
 }
 
 // Half of a Heun step: stage 1, or stage 2 with the end-of-step bookkeeping
-// (tau advance, rotation of the primitive sets).
+// (tau, which its last kernel advanced on the device, and the rotation of the primitive sets).
 template <typename R, bool VISC>
 void launch_half(clv_handle* h, int stage, bool stats, bool timed) {
   if (stage == 1) {
@@ -602,7 +589,6 @@ void launch_half(clv_handle* h, int stage, bool stats, bool timed) {
     launch_stage<R, VISC, 2, false>(h, p2, timed);
   }
   if (h->charge_on) launch_charge_stage<R>(p2, 2, h->NC[1], h->NC[0], h->NC[0], h->stream);
-  advance_tau_kernel<<<1, 1, 0, h->stream>>>(h->tau_dev, h->itau_dev, h->cfg.dtau, h->cfg.cartesian);
   std::swap(h->cur, h->prev);
   h->tau = h->tau + h->cfg.dtau;
   h->step += 1;
@@ -747,10 +733,29 @@ template <typename R> clv_status reduce_stats(clv_handle* h, bool scan, clv_stat
   return CLV_OK;
 }
 
-// compact doubles -> the padded layout in R
-template <typename R> __global__ void convert_kernel(const double* s, R* d, long long N, int ne, int nep) {
+// compact doubles -> the padded layout in R, field blockIdx.y (padding slots
+// and fields without a source: 0)
+constexpr int kMaxConvert = 14;
+template <typename R> struct ConvertSet {
+  const double* s[kMaxConvert];
+  R* d[kMaxConvert];
+};
+template <typename R>
+__global__ void __launch_bounds__(kBlock) convert_kernel(const ConvertSet<R> x, long long npad, int ne, int nep) {
   const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (c < N) d[padded_index(c, ne, nep)] = (R)s[c];
+  if (c >= npad) return;
+  const double* s = x.s[blockIdx.y];
+  long long row;
+  int k;
+  if (npad <= (1ll << 31)) {
+    const unsigned r = (unsigned)c / (unsigned)nep;
+    row = r;
+    k = (int)((unsigned)c - r * (unsigned)nep);
+  } else {
+    row = c / nep;
+    k = (int)(c - row * nep);
+  }
+  x.d[blockIdx.y][c] = s && k < ne ? (R)s[row * ne + k] : R(0);
 }
 
 template <typename R> Prim<R> prim_at(Prim<R> p, long long off) {
@@ -769,35 +774,39 @@ template <typename R> Prim<R> prim_at(Prim<R> p, long long off) {
 template <typename R>
 clv_status load_initial_range(clv_handle* h, long long off, long long npad, long long nc, int ne, int nep, bool visc,
                               const double* const in[4], const double* pi, bool host) {
-  const unsigned gc = grid_of(nc), gp = grid_of(npad);
+  const unsigned gp = grid_of(npad);
   const clv_config& c = h->cfg;
   Prim<R> pc = prim_at(prim_set<R>(h, h->cur), off), pp = prim_at(prim_set<R>(h, h->prev), off);
-  R* dst_prim[4] = {pc.e, pc.u[0], pc.u[1], pc.u[2]};
-  for (int f = 0; f < 4; ++f) {
-    const double* src = in[f];
-    if (host) {
-      CLV_CUDA(h, cudaMemcpyAsync(h->staging, src, (size_t)nc * 8, cudaMemcpyHostToDevice, h->stream));
-      src = h->staging;
-    }
-    if (nep != ne) CLV_CUDA(h, cudaMemsetAsync(dst_prim[f], 0, (size_t)npad * sizeof(R), h->stream));
-    convert_kernel<R><<<gc, kBlock, 0, h->stream>>>(src, dst_prim[f], nc, ne, nep);
-  }
   Ptr10<R> pi0;
   for (int q = 0; q < 10; ++q) pi0.p[q] = (R*)h->PI0[q] + off;
-  for (int q = 0; q < 10; ++q) {
-    CLV_CUDA(h, cudaMemsetAsync(pi0.p[q], 0, (size_t)npad * sizeof(R), h->stream));
-    if (pi && visc) {
-      const double* src = pi + (size_t)q * nc;
-      if (host) {
-        CLV_CUDA(h, cudaMemcpyAsync(h->staging, src, (size_t)nc * 8, cudaMemcpyHostToDevice, h->stream));
-        src = h->staging;
-      }
-      convert_kernel<R><<<gc, kBlock, 0, h->stream>>>(src, pi0.p[q], nc, ne, nep);
+  // eps, u~, pi~: sources on the device in one launch; host arrays one at a
+  // time through the staging buffer
+  ConvertSet<R> all{};
+  for (int f = 0; f < kMaxConvert; ++f) {
+    all.d[f] = f == 0 ? pc.e : f < 4 ? pc.u[f - 1] : pi0.p[f - 4];
+    all.s[f] = f < 4 ? in[f] : pi && visc ? pi + (size_t)(f - 4) * nc : nullptr;
+    if (!host) continue;
+    ConvertSet<R> one{};
+    one.d[0] = all.d[f];
+    if (all.s[f]) {
+      CLV_CUDA(h, cudaMemcpyAsync(h->staging, all.s[f], (size_t)nc * 8, cudaMemcpyHostToDevice, h->stream));
+      one.s[0] = h->staging;
     }
+    convert_kernel<R><<<gp, kBlock, 0, h->stream>>>(one, npad, ne, nep);
   }
+  if (!host) convert_kernel<R><<<dim3(gp, kMaxConvert), kBlock, 0, h->stream>>>(all, npad, ne, nep);
   init_primitives_kernel<R><<<gp, kBlock, 0, h->stream>>>(pc, pp, pi0, visc, eos_view<R>(h), c.eps_cut, npad);
   CLV_CUDA(h, cudaGetLastError());
   return CLV_OK;
+}
+
+// zeros in the stage-2 shear buffers, halo planes included (the ten arrays
+// follow one another in the workspace, layout())
+cudaError_t clear_stage_shear(clv_handle* h) {
+  const size_t halo = (size_t)h->cfg.halo_x * h->cfg.ny * h->nep * h->rsize;
+  char* first = (char*)h->PI1[0] - halo;
+  char* end = (char*)h->PI1[9] + (size_t)h->N * h->rsize + halo;
+  return cudaMemsetAsync(first, 0, (size_t)(end - first), h->stream);
 }
 
 // The rest of the initial state, over all cells: tau reset and T~ from the
@@ -811,7 +820,7 @@ template <typename R> clv_status initial_begin(clv_handle* h) {
   Ptr10<R> pi0;
   for (int q = 0; q < 10; ++q) pi0.p[q] = (R*)h->PI0[q];
   if (!h->batch.empty())   // ideal events of a batch keep pi~ = 0 in the stage buffers too
-    for (int q = 0; q < 10; ++q) CLV_CUDA(h, cudaMemsetAsync(h->PI1[q], 0, (size_t)N * sizeof(R), h->stream));
+    CLV_CUDA(h, clear_stage_shear(h));
   const double taus0 = c.cartesian ? 1.0 : c.tau0;
   set_tau(h, c.tau0);
   h->step = 0;
@@ -874,16 +883,9 @@ clv_status set_initial_impl(clv_handle* h, const double* const in[4], const doub
   return s != CLV_OK ? s : finish_initial<R>(h);
 }
 
-// field `which` of the grid at padded offset off (n compact cells, eta rows
-// ne of pitch nep) as compact doubles
-template <typename R>
-clv_status export_field(clv_handle* h, int which, double* dst, long long off, long long n, int ne, int nep) {
-  if (which == 22) {   // n = N~^tau / (tau u~^tau)
-    launch_charge_density<R>(h->NC[0], prim_set<R>(h, h->cur), h->cfg.cartesian ? 1.0 : h->tau, dst, n, ne, nep,
-                             h->stream);
-    CLV_CUDA(h, cudaGetLastError());
-    return CLV_OK;
-  }
+// Source of field `which` (not 22) at padded offset off: high parts and, for
+// the T~ of the FP32 path, low parts.
+template <typename R> void field_source(clv_handle* h, int which, long long off, const R*& hi, const R*& lo) {
   const void* src = nullptr;
   if (which <= 3) src = h->PR[h->cur][which];
   else if (which <= 7) src = h->T0[which - 4];
@@ -891,11 +893,29 @@ clv_status export_field(clv_handle* h, int which, double* dst, long long off, lo
   else if (which <= 20) src = h->PR[h->prev][1 + (which - 18)];
   else if (which == 23) src = h->PB[0];
   else src = h->NC[0];
-  if (which >= 4 && which <= 7 && h->TL0[0])   // FP32 path: T~ = high + low parts
-    export_pair_kernel<R><<<grid_of(n), kBlock, 0, h->stream>>>((const R*)src + off,
-                                                                (const R*)h->TL0[which - 4] + off, dst, n, ne, nep);
-  else
-    export_kernel<R><<<grid_of(n), kBlock, 0, h->stream>>>((const R*)src + off, dst, n, ne, nep);
+  hi = (const R*)src + off;
+  lo = which >= 4 && which <= 7 && h->TL0[0] ? (const R*)h->TL0[which - 4] + off : nullptr;
+}
+
+// Fields `which[0 .. nf)` of the grid at padded offset off (n compact cells,
+// eta rows ne of pitch nep) as compact doubles, field i to dst + i n: one
+// launch for all but n = N~^tau / (tau u~^tau) (field 22).
+template <typename R>
+clv_status export_fields(clv_handle* h, const int* which, int nf, double* dst, long long off, long long n, int ne,
+                         int nep) {
+  ExportSet<R> x{};
+  int m = 0;
+  for (int i = 0; i < nf; ++i) {
+    double* d = dst + (size_t)i * (size_t)n;
+    if (which[i] == 22) {
+      launch_charge_density<R>(h->NC[0], prim_set<R>(h, h->cur), h->cfg.cartesian ? 1.0 : h->tau, d, n, ne, nep,
+                               h->stream);
+      continue;
+    }
+    field_source<R>(h, which[i], off, x.hi[m], x.lo[m]);
+    x.dst[m++] = d;
+  }
+  if (m) export_kernel<R><<<dim3(grid_of(n), (unsigned)m), kBlock, 0, h->stream>>>(x, n, ne, nep);
   CLV_CUDA(h, cudaGetLastError());
   return CLV_OK;
 }
@@ -1077,10 +1097,7 @@ static clv_status set_initial_T_any(clv_handle* h, const double* T, bool host) {
   if (st != CLV_OK) return st;
   // the scratch is consumed (stream order): the stage buffers return to zeros, as the
   // padding slots of the eta rows, which the stages never write, must stay vacuum
-  for (int q = 0; q < 10; ++q)
-    CLV_CUDA(h, cudaMemsetAsync((char*)h->PI1[q] - (size_t)h->cfg.halo_x * h->cfg.ny * h->nep * h->rsize, 0,
-                                ((size_t)h->N + 2 * (size_t)h->cfg.halo_x * h->cfg.ny * h->nep) * h->rsize,
-                                h->stream));
+  CLV_CUDA(h, clear_stage_shear(h));
   return CLV_OK;
 }
 
@@ -1181,19 +1198,20 @@ static clv_status get_fields_range(clv_handle* h, uint32_t mask, double* out, bo
   if (mask >> 24) return fail(h, CLV_EINVAL, "mask selects fields beyond index 23");
   if ((mask >> 21 & 3u) && !h->cfg.charge) return fail(h, CLV_EINVAL, "fields 21 and 22 need charge = 1");
   if ((mask >> 23 & 1u) && !h->PB[0]) return fail(h, CLV_EINVAL, "field 23 needs zeta_over_s > 0");
-  size_t slot = 0;
-  for (int f = 0; f < 24; ++f) {
-    if (!(mask >> f & 1u)) continue;
-    double* dst = host ? h->staging : out + slot * (size_t)n;
-    clv_status s = h->rsize == 8 ? export_field<double>(h, f, dst, off, n, ne, nep)
-                                 : export_field<float>(h, f, dst, off, n, ne, nep);
+  int which[kMaxExport], nf = 0;
+  for (int f = 0; f < kMaxExport; ++f)
+    if (mask >> f & 1u) which[nf++] = f;
+  auto fields = [&](const int* w, int m, double* dst) {
+    return h->rsize == 8 ? export_fields<double>(h, w, m, dst, off, n, ne, nep)
+                         : export_fields<float>(h, w, m, dst, off, n, ne, nep);
+  };
+  if (!host) return nf ? fields(which, nf, out) : CLV_OK;
+  for (int i = 0; i < nf; ++i) {   // host arrays one at a time through the staging buffer
+    const clv_status s = fields(which + i, 1, h->staging);
     if (s != CLV_OK) return s;
-    if (host) {
-      CLV_CUDA(h, cudaMemcpyAsync(out + slot * (size_t)n, h->staging, (size_t)n * 8,
-                                  cudaMemcpyDeviceToHost, h->stream));
-      CLV_CUDA(h, cudaStreamSynchronize(h->stream));
-    }
-    ++slot;
+    CLV_CUDA(h, cudaMemcpyAsync(out + (size_t)i * (size_t)n, h->staging, (size_t)n * 8, cudaMemcpyDeviceToHost,
+                                h->stream));
+    CLV_CUDA(h, cudaStreamSynchronize(h->stream));
   }
   return CLV_OK;
 }

@@ -65,6 +65,7 @@ template <typename R, int STAGE>
 __global__ void __launch_bounds__(kBlock) bulk_stage_kernel(const StageParams<R> p, const R* __restrict__ Pin,
                                                             const R* Pn, R* Pout,   // Pn == Pout in stage 2
                                                             const R inv_5zs_hbarc) {
+  enter_step_kernel();
   const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= p.N) return;
   const int k = (int)(c % p.nep);
@@ -121,9 +122,9 @@ void launch_bulk_stage(const StageParams<R>& p, int stage, const void* Pin, cons
   const unsigned g = (unsigned)((p.N + kBlock - 1) / kBlock);
   const R coef = (R)(1.0 / (5.0 * zeta_over_s * kHbarcBulk));
   if (stage == 1)
-    bulk_stage_kernel<R, 1><<<g, kBlock, 0, st>>>(p, (const R*)Pin, (const R*)Pn, (R*)Pout, coef);
+    launch_step_kernel(bulk_stage_kernel<R, 1>, g, kBlock, 0, st, p, (const R*)Pin, (const R*)Pn, (R*)Pout, coef);
   else
-    bulk_stage_kernel<R, 2><<<g, kBlock, 0, st>>>(p, (const R*)Pin, (const R*)Pn, (R*)Pout, coef);
+    launch_step_kernel(bulk_stage_kernel<R, 2>, g, kBlock, 0, st, p, (const R*)Pin, (const R*)Pn, (R*)Pout, coef);
 }
 
 template void launch_bulk_stage<float>(const StageParams<float>&, int, const void*, const void*, void*, double,

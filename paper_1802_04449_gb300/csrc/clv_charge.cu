@@ -49,6 +49,7 @@ __device__ __forceinline__ R charge_flux(const ChargeCell<R>& a, const ChargeCel
 template <typename R, int STAGE>
 __global__ void __launch_bounds__(kBlock) charge_stage_kernel(const StageParams<R> p, const R* __restrict__ Nin,
                                                               const R* Nn, R* Nout) {   // Nn == Nout in stage 2
+  enter_step_kernel();
   const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= p.N) return;
   const int k = (int)(c % p.nep);
@@ -107,9 +108,9 @@ void launch_charge_stage(const StageParams<R>& p, int stage, const void* Nin, co
                          cudaStream_t st) {
   const unsigned g = (unsigned)((p.N + kBlock - 1) / kBlock);
   if (stage == 1)
-    charge_stage_kernel<R, 1><<<g, kBlock, 0, st>>>(p, (const R*)Nin, (const R*)Nn, (R*)Nout);
+    launch_step_kernel(charge_stage_kernel<R, 1>, g, kBlock, 0, st, p, (const R*)Nin, (const R*)Nn, (R*)Nout);
   else
-    charge_stage_kernel<R, 2><<<g, kBlock, 0, st>>>(p, (const R*)Nin, (const R*)Nn, (R*)Nout);
+    launch_step_kernel(charge_stage_kernel<R, 2>, g, kBlock, 0, st, p, (const R*)Nin, (const R*)Nn, (R*)Nout);
 }
 
 template <typename R>

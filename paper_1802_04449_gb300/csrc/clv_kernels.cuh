@@ -39,6 +39,22 @@ template <typename R> struct IsCoef {
 // sources stay FP32); the update adds the FP32 increment to the pair exactly,
 // and the recovery forms E and M from the pair.  The FP64 path stores T~ in
 // T and leaves Tl unused.
+// tau of a step and 1/tau of its end (tau + dtau; 1 in Cartesian mode) as a
+// float-float pair for the FP32 recovery.  A handle has two, used by alternate
+// steps like the primitive sets: the last kernel of a step writes the next
+// one's while its own is still being read.
+struct TauSlot {
+  double tau;
+  float itau[2];
+};
+__device__ __forceinline__ void store_tau(TauSlot* s, double tau, double dtau, int cartesian) {
+  const double x = cartesian ? 1.0 : 1.0 / (tau + dtau);
+  const float hi = (float)x;
+  s->tau = tau;
+  s->itau[0] = hi;
+  s->itau[1] = (float)(x - (double)hi);
+}
+
 template <typename R> struct StageParams {
   // fields of the stage being differentiated (stage 1: step n, stage 2: stage-1 result)
   const R* T[4];
@@ -66,6 +82,7 @@ template <typename R> struct StageParams {
   // replays unchanged; tau_scalars() forms the stage's tau factors from it
   const double* tau_dev;
   const float* itau;   // FP32 path: 1/tau at the end of the step (Cartesian: 1) as a float-float pair
+  TauSlot* tau_next;   // stage 2: tau of the next step, written by the root solve (nullptr in stage 1)
   double dtau_d;
   int cartesian;
   // scalars in the working precision
@@ -94,6 +111,30 @@ template <typename R> struct StageParams {
 // kGuessMlp: the network seeds the cells that were vacuum in the stage's
 // input (no velocity to start from), the stage velocity every other cell;
 // kGuessMlpAll: the network seeds every cell.
+// Kernels of a step start while their predecessor drains (programmatic
+// dependent launch): the next one may be placed as soon as every CTA of this
+// one runs, and nothing of this one is done before its predecessor is complete
+// and its writes visible.  No effect on a plain launch.
+__device__ __forceinline__ void enter_step_kernel() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <typename... P, typename... A>
+inline void launch_step_kernel(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st,
+                               const A&... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3(grid);
+  c.blockDim = dim3(block);
+  c.dynamicSmemBytes = smem;
+  c.stream = st;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  cudaLaunchKernelEx(&c, kernel, P(args)...);   // an error is left for cudaGetLastError, as by <<<>>>
+}
+
 enum GuessMode { kGuessPrevious = 0, kGuessCold = 1, kGuessMlp = 2, kGuessMlpAll = 3 };
 
 __device__ __forceinline__ int wrap_index(int i, int n, int periodic) {
@@ -402,6 +443,7 @@ __device__ __forceinline__ void shear_source(R geo, const R u[4], R du[4][4], co
 
 template <typename R, int STAGE, bool VISC, bool STATS>
 __global__ void __launch_bounds__(kBlock) stage_kernel(const StageParams<R> p) {
+  enter_step_kernel();
   const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const bool active = c < p.N && (int)(c % p.nep) < p.ne;   // padding slots of the eta rows do no work
   double my_T0 = 0.0;
@@ -642,6 +684,7 @@ __global__ void __launch_bounds__(kBlock) stage_kernel(const StageParams<R> p) {
     my_T0 = (double)Tnew[0] + (sizeof(R) == 4 ? (double)Tnl[0] : 0.0);
     my_e = (double)en;
   }
+  if (STAGE == 2 && c == 0) store_tau(p.tau_next, *p.tau_dev + p.dtau_d, p.dtau_d, p.cartesian);
   // ---------------- counters and reductions ----------------
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
@@ -691,6 +734,7 @@ struct RecoverMinBlocks {
 
 template <typename R, bool VISC, bool STATS, int GUESS = kGuessPrevious>
 __global__ void __launch_bounds__(kBlock, RecoverMinBlocks<R>::value) recover_kernel(const StageParams<R> p) {
+  enter_step_kernel();
   const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const bool active = c < p.N;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -852,6 +896,7 @@ __global__ void __launch_bounds__(kBlock, RecoverMinBlocks<R>::value) recover_ke
     my_T0 = T0v;
     my_e = (double)en;
   }
+  if (p.tau_next && c == 0) store_tau(p.tau_next, *p.tau_dev + p.dtau_d, p.dtau_d, p.cartesian);
   const unsigned full = 0xffffffffu;
   const unsigned b_res = __ballot_sync(full, f_rescaled);
   const unsigned b_fail = __ballot_sync(full, f_fail);
@@ -1057,24 +1102,29 @@ __global__ void __launch_bounds__(kBlock) extrapolate_prev_kernel(Prim<R> cur, P
 // Cell c of the compact order (nx, ny, neta) <-> its slot in the padded
 // layout, whose eta rows have a pitch nep >= neta (a multiple of 4).
 __device__ __forceinline__ long long padded_index(long long c, int ne, int nep) {
+  if (c < (1ll << 31)) {   // 32-bit division
+    const unsigned row = (unsigned)c / (unsigned)ne;
+    return (long long)row * nep + ((unsigned)c - row * (unsigned)ne);
+  }
   return (c / ne) * nep + c % ne;
 }
 
+// fields as compact doubles, field blockIdx.y to dst + blockIdx.y N; a
+// float-float field is the sum of its high and low parts (lo: else nullptr)
+constexpr int kMaxExport = 24;
+template <typename R> struct ExportSet {
+  const R *hi[kMaxExport], *lo[kMaxExport];
+  double* dst[kMaxExport];
+};
 template <typename R>
-__global__ void __launch_bounds__(kBlock) export_kernel(const R* src, double* dst, long long N, int ne, int nep) {
+__global__ void __launch_bounds__(kBlock) export_kernel(const ExportSet<R> x, long long N, int ne, int nep) {
   const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (c < N) dst[c] = (double)src[padded_index(c, ne, nep)];
-}
-
-// a float-float field (high and low parts) as compact doubles
-template <typename R>
-__global__ void __launch_bounds__(kBlock) export_pair_kernel(const R* hi, const R* lo, double* dst, long long N, int ne,
-                                                             int nep) {
-  const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (c < N) {
-    const long long k = padded_index(c, ne, nep);
-    dst[c] = (double)hi[k] + (double)lo[k];
-  }
+  if (c >= N) return;
+  const long long k = padded_index(c, ne, nep);
+  const R *hi = x.hi[blockIdx.y], *lo = x.lo[blockIdx.y];
+  double v = (double)hi[k];
+  if (lo) v += (double)lo[k];
+  x.dst[blockIdx.y][c] = v;
 }
 
 // Deterministic final sum of the per-block partials (one block).

@@ -567,6 +567,7 @@ __device__ __forceinline__ void stage_tile_body(const StageParams<R>& p, const E
 template <typename R, int STAGE, bool VISC>
 __global__ void __launch_bounds__(TileBound<R>::threads, 1)
     stage_tile_kernel(const StageParams<R> p, const TileArgs t) {
+  enter_step_kernel();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const EventGeom<R> ev{0, p.nx, p.ny, p.ne, p.nep, p.inv_dl[0], p.inv_dl[1], p.is, p.deta_d, VISC ? 1 : 0};
   stage_tile_body<R, STAGE, VISC>(p, ev, t, blockIdx.x, smem_raw);
@@ -581,6 +582,7 @@ template <typename R, int STAGE, bool ANY_VISC>
 __global__ void __launch_bounds__(TileBound<R>::threads, 1)
     stage_batch_kernel(const StageParams<R> p, const EventGeom<R>* __restrict__ evs,
                        const TileArgs* __restrict__ tiles, const int2* __restrict__ items, int nitems, int* next) {
+  enter_step_kernel();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int s_item;
   for (;;) {
