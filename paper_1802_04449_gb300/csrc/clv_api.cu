@@ -318,6 +318,8 @@ std::vector<TileGeom> tile_candidates(const clv_config* c, int sms, size_t smem_
   return out;
 }
 
+constexpr int kRecoverSmall = 64;   // threads of a recovery block on a small grid (recover_block)
+
 inline int eta_pitch(int neta) { return (neta + 3) & ~3; }
 
 size_t layout(const clv_config* c, clv_handle* h) {
@@ -332,9 +334,8 @@ size_t layout(const clv_config* c, clv_handle* h) {
   const size_t fb = align_up((size_t)N * rs + 2 * hoff, 256);
   // FP32 path: T~ as float-float pairs (StageParams), the low parts in 2 x 4 more arrays
   const bool ffT = c->precision != CLV_FP64;
-  // block partials of the stats reduction: enough for the direct grid and for
-  // the tiled grid on any device (at most 1024 SMs)
-  const int nblocks = (int)std::max<long long>((N + kBlock - 1) / kBlock, tile_geometry(c, 1024).blocks);
+  // block partials of the stats reduction: enough for the smallest recovery blocks
+  const int nblocks = (int)((N + kRecoverSmall - 1) / kRecoverSmall);
   size_t off = 0;
   auto take = [&](size_t bytes) { size_t o = off; off += align_up(bytes, 256); return o; };
   size_t oT0[4], oPI0[10], oT1[4], oPI1[10], oPR[kNumPrimSets][kPrimFields], oE[3];
@@ -519,14 +520,23 @@ template <typename R, bool VISC> cudaError_t tile_attributes(size_t smem) {
   return e;
 }
 
+// Threads of a recovery block: kBlock, or kRecoverSmall on a grid that would
+// not give every SM a block of kBlock (the cells of 33 x 33 x 9: 20 us with 52
+// blocks of 256 on 152 SMs in FP64, whose pipe is what the solve waits for).
+inline int recover_block(const clv_handle* h) { return (h->N + kBlock - 1) / kBlock < 2ll * h->sms ? kRecoverSmall : kBlock; }
+inline unsigned recover_grid(const clv_handle* h) {
+  const int b = recover_block(h);
+  return (unsigned)((h->N + b - 1) / b);
+}
+
 template <typename R, bool VISC, bool STATS> void launch_recover(clv_handle* h, const StageParams<R>& p) {
-  const unsigned g = grid_of(h->N);
+  const unsigned g = recover_grid(h), b = (unsigned)recover_block(h);
   if (sizeof(R) == 4 && h->guess == kGuessMlp)
-    launch_step_kernel(recover_kernel<R, VISC, STATS, sizeof(R) == 4 ? kGuessMlp : kGuessPrevious>, g, kBlock, 0, h->stream, p);
+    launch_step_kernel(recover_kernel<R, VISC, STATS, sizeof(R) == 4 ? kGuessMlp : kGuessPrevious>, g, b, 0, h->stream, p);
   else if (sizeof(R) == 4 && h->guess == kGuessMlpAll)
-    launch_step_kernel(recover_kernel<R, VISC, STATS, sizeof(R) == 4 ? kGuessMlpAll : kGuessPrevious>, g, kBlock, 0, h->stream, p);
-  else if (h->guess == kGuessCold) launch_step_kernel(recover_kernel<R, VISC, STATS, kGuessCold>, g, kBlock, 0, h->stream, p);
-  else launch_step_kernel(recover_kernel<R, VISC, STATS, kGuessPrevious>, g, kBlock, 0, h->stream, p);
+    launch_step_kernel(recover_kernel<R, VISC, STATS, sizeof(R) == 4 ? kGuessMlpAll : kGuessPrevious>, g, b, 0, h->stream, p);
+  else if (h->guess == kGuessCold) launch_step_kernel(recover_kernel<R, VISC, STATS, kGuessCold>, g, b, 0, h->stream, p);
+  else launch_step_kernel(recover_kernel<R, VISC, STATS, kGuessPrevious>, g, b, 0, h->stream, p);
 }
 
 // One stage: the stage kernel, then the root solve (the direct kernel does
@@ -584,7 +594,7 @@ void launch_half(clv_handle* h, int stage, bool stats, bool timed) {
   }
   if (stats) {
     launch_stage<R, VISC, 2, true>(h, p2, timed);
-    h->stat_blocks = (int)grid_of(h->N);
+    h->stat_blocks = (int)(h->batch.empty() && h->cfg.kernel == 1 ? grid_of(h->N) : recover_grid(h));
   } else {
     launch_stage<R, VISC, 2, false>(h, p2, timed);
   }

@@ -737,7 +737,7 @@ __global__ void __launch_bounds__(kBlock, RecoverMinBlocks<R>::value) recover_ke
   enter_step_kernel();
   const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const bool active = c < p.N;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
   double my_T0 = 0.0, my_e = 0.0;
   int my_iters = 0, my_solved = 0, my_polish_iters = 0;
   bool f_rescaled = false, f_fail = false, f_polished = false, f_nonfinite = false, f_nonconv = false;
@@ -928,7 +928,8 @@ __global__ void __launch_bounds__(kBlock, RecoverMinBlocks<R>::value) recover_ke
   if (threadIdx.x < 9) {
     unsigned long long t = 0;
 #pragma unroll
-    for (int w = 0; w < kBlock / 32; ++w) t += s_cnt[w][threadIdx.x];
+    for (int w = 0; w < kBlock / 32; ++w)
+      if (w < nwarp) t += s_cnt[w][threadIdx.x];
     if (t) atomicAdd(p.counters + threadIdx.x, t);
   }
   if constexpr (STATS) {
@@ -944,7 +945,7 @@ __global__ void __launch_bounds__(kBlock, RecoverMinBlocks<R>::value) recover_ke
     __syncthreads();
     if (threadIdx.x == 0) {
       double a = 0.0, b = 0.0;
-      for (int w = 0; w < kBlock / 32; ++w) { a += s_sum[w]; b = fmax(b, s_max[w]); }
+      for (int w = 0; w < nwarp; ++w) { a += s_sum[w]; b = fmax(b, s_max[w]); }
       p.block_sum[blockIdx.x] = a;
       if (b > 0.0) atomicMax(p.emax_bits, (unsigned long long)__double_as_longlong(b));
     }
