@@ -214,54 +214,51 @@ int kernel_occupancy(const void* f, int threads, size_t smem) {
   return std::max(1, n);
 }
 
+// CTAs of a tile on one SM by its shared memory and registers (168 a thread in
+// FP32, 255 in FP64, as the launch bounds leave them)
 int tile_occupancy(const clv_config* c, int threads, size_t smem) {
-  const bool visc = c->eta_over_s > 0.0;
-  if (c->precision == CLV_FP64)
-    return kernel_occupancy(visc ? (const void*)stage_tile_kernel<double, 2, true> : (const void*)stage_tile_kernel<double, 2, false>,
-                            threads, smem);
-  return kernel_occupancy(visc ? (const void*)stage_tile_kernel<float, 2, true> : (const void*)stage_tile_kernel<float, 2, false>,
-                          threads, smem);
+  const int warps = (threads + 31) / 32, regs = (c->precision == CLV_FP64 ? 256 : 168) * 32;
+  const int by_regs = 65536 / (warps * regs), by_smem = (int)(233472 / (smem + 1024));
+  return std::max(1, std::min({by_regs, by_smem, 2048 / (32 * warps)}));
 }
 
+// Modelled time of a plane of one CTA with occ CTAs on its SM, and the planes
+// that a chunk costs beyond its own.  FP32: a plane is a chain of ~2000
+// dependent instructions whatever the tile, plus the box's cells (97 x 97 x 41
+// viscous stage 1: 7 x 22 tiles 4.8 us, 12 x 21 5.3, 16 x 21 6.0, two of 7 x 21
+// 5.8); the 4 halo planes, without y and eta interfaces, cost about 3.  FP64:
+// the cells and their halo on the FP64 pipe over a chain that is the longer
+// part of an ideal tile (33 x 33 x 9: 18 x 9 tiles 41 us, 9 x 9 35, 3 x 9 with
+// three planes 59; 97 x 97 x 41 viscous: 7 x 21 and 10 x 14 1.11 ms, 4 x 21
+// 1.35, 7 x 14 in two waves 1.24).
+double plane_cost(const clv_config* c, int TJ, int TK, int occ) {
+  if (c->precision == CLV_FP64) return (c->eta_over_s > 0.0 ? 200.0 : 435.0) + occ * (double)((TJ + 2) * (TK + 2));
+  return 620.0 + occ * (double)((TJ + 4) * box_width(TK));
+}
+inline double halo_planes(const clv_config* c) { return c->precision == CLV_FP64 ? 1.2 : 3.0; }
+
 // x chunking of a tile grid: the number of chunks that minimises waves x
-// (planes per chunk + the 4 halo planes each chunk also stages), with `slots`
-// CTAs resident on the device at a time
-int chunk_planes(int nx, long long tiles, long long slots) {
+// (planes per chunk + the cost of its halo planes), with `slots` CTAs resident
+// on the device at a time
+int chunk_planes(int nx, long long tiles, long long slots, double halo) {
   long long best_nch = 1;
   double best = 1e300;
   for (long long nch = 1; nch <= std::min<long long>(nx, 8LL * slots); ++nch) {
     const long long cx = (nx + nch - 1) / nch;
     const long long used = (nx + cx - 1) / cx;
     const long long waves = (tiles * used + slots - 1) / slots;
-    const double cost = (double)waves * (double)(cx + 4);
+    const double cost = (double)waves * ((double)cx + halo);
     if (cost < best - 1e-9) { best = cost; best_nch = used; }
   }
   return (int)((nx + best_nch - 1) / best_nch);
 }
 
-TileGeom tile_geometry_of(const clv_config* c, int sms, int TJ, int TK, int cx);
-
-// Tile shape: TK columns fit neta in ceil(neta/32) tiles; the block has
-// (TJ+1) x (TK+1) threads, at most CLV_TILE_MAX_THREADS (FP32) or 128 (FP64),
-// and fewer rows while its shared memory exceeds the opt-in limit of a block;
-// x is cut into chunks of CX planes by the makespan rule of chunk_planes.
-TileGeom tile_geometry(const clv_config* c, int sms) {
-  const int rsize = c->precision == CLV_FP64 ? 8 : 4;
-  const int maxthr = rsize == 4 ? CLV_TILE_MAX_THREADS : std::min(CLV_TILE_MAX_THREADS, kBlock / 2);
-  const int nk = (c->neta + 31) / 32;
-  const int TK = (c->neta + nk - 1) / nk;
-  const bool visc = c->eta_over_s > 0.0;
-  int TJ = std::max(1, std::min(c->ny, maxthr / (TK + 1) - 1));
-  auto smem_of = [&](int tj) {
-    return visc ? tile_smem_bytes<true>(tj, TK, rsize) : tile_smem_bytes<false>(tj, TK, rsize);
-  };
-  while (TJ > 1 && smem_of(TJ) > kSmemOptinMax) --TJ;
-  return tile_geometry_of(c, sms, TJ, TK, 0);
+inline int tile_max_threads(const clv_config* c) {
+  return c->precision == CLV_FP64 ? TileBound<double>::threads : TileBound<float>::threads;
 }
 
 // Geometry of an explicit (TJ, TK) tile shape; CX from the makespan rule of
-// chunk_planes when cx <= 0, with as many CTAs per SM as the device keeps
-// resident at this shape.
+// chunk_planes when cx <= 0, with as many CTAs per SM as fit at this shape.
 TileGeom tile_geometry_of(const clv_config* c, int sms, int TJ, int TK, int cx) {
   const int rsize = c->precision == CLV_FP64 ? 8 : 4;
   TileGeom g;
@@ -274,28 +271,22 @@ TileGeom tile_geometry_of(const clv_config* c, int sms, int TJ, int TK, int cx) 
   g.threads = (TJ + 1) * (TK + 1);
   g.smem = visc ? tile_smem_bytes<true>(TJ, TK, rsize) : tile_smem_bytes<false>(TJ, TK, rsize);
   const long long tiles = (long long)t.ntj * t.ntk;
-  if (cx <= 0) cx = chunk_planes(c->nx, tiles, (long long)sms * tile_occupancy(c, g.threads, g.smem));
+  if (cx <= 0) cx = chunk_planes(c->nx, tiles, (long long)sms * tile_occupancy(c, g.threads, g.smem), halo_planes(c));
   t.CX = cx;
   const long long nch = (c->nx + t.CX - 1) / t.CX;
   g.blocks = (unsigned)(tiles * nch);
   return g;
 }
 
-inline int tile_max_threads(const clv_config* c) {
-  return c->precision == CLV_FP64 ? std::min(CLV_TILE_MAX_THREADS, kBlock / 2) : CLV_TILE_MAX_THREADS;
-}
-
-// Candidate tile shapes for the autotuner, best modelled makespan first:
-// eta_s split into 1..4 columns of tiles, y tiles from the largest that fits
-// the thread limit down to a third of it, the x chunking of each by the
-// makespan rule.  Model: waves x (planes + 4 halo planes) x staged box cells
-// x CTAs sharing an SM, over the SM's issue efficiency (resident warps, up to
-// 16, over 16).
+// Tile shapes by modelled makespan, the best first: waves x (planes + halo
+// planes) x plane_cost.  eta_s split into 1..4 columns of tiles or into columns
+// of at most 32, y tiles from the largest that fits the thread limit down to a
+// third of it, the x chunking of each by the makespan rule.
 std::vector<TileGeom> tile_candidates(const clv_config* c, int sms, size_t smem_max) {
   std::vector<std::pair<double, TileGeom>> v;
   const int maxthr = tile_max_threads(c);
   int last_tk = -1;
-  for (int nk = 1; nk <= 4; ++nk) {
+  for (int nk = 1; nk <= std::max(4, (c->neta + 31) / 32); nk = nk == 4 ? std::max(5, (c->neta + 31) / 32) : nk + 1) {
     const int TK = (c->neta + nk - 1) / nk;
     if (TK == last_tk || TK < 1) continue;
     last_tk = TK;
@@ -307,15 +298,21 @@ std::vector<TileGeom> tile_candidates(const clv_config* c, int sms, size_t smem_
       const int occ = tile_occupancy(c, g.threads, g.smem);
       const long long slots = (long long)sms * occ;
       const long long waves = ((long long)g.blocks + slots - 1) / slots;
-      const double eff = std::min(1.0, occ * ((g.threads + 31) / 32) / 16.0);
-      const double cost = (double)waves * (g.t.CX + 4) * (double)((TJ + 4) * (TK + 4)) * occ / eff;
-      v.push_back({cost, g});
+      v.push_back({(double)waves * (g.t.CX + halo_planes(c)) * plane_cost(c, TJ, TK, occ), g});
     }
   }
   std::stable_sort(v.begin(), v.end(), [](const auto& a, const auto& b) { return a.first < b.first; });
   std::vector<TileGeom> out;
   for (auto& x : v) out.push_back(x.second);
   return out;
+}
+
+// Default tile shape: the best candidate of the model (97 x 97 x 41 in FP32: 8
+// x 41 cells, 70 us a stage 1; the largest tile of two eta columns, 16 x 21,
+// took 80).  A tile of one cell always fits.
+TileGeom tile_geometry(const clv_config* c, int sms) {
+  const std::vector<TileGeom> v = tile_candidates(c, sms, kSmemOptinMax);
+  return v.empty() ? tile_geometry_of(c, sms, 1, 1, 0) : v.front();
 }
 
 constexpr int kRecoverSmall = 64;   // threads of a recovery block on a small grid (recover_block)

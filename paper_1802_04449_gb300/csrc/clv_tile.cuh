@@ -207,12 +207,13 @@ __device__ __forceinline__ void box_interface(const R* box, int NB, int c, int s
 // Thread cap of a stage-kernel CTA.  FP32: 384 threads (12 warps) fit the
 // register file at the 168 registers that bound allows; a CTA of at most 192
 // threads then leaves room for a second one on the SM, when its shared
-// memory fits too.  FP64: 128 threads (255 registers).
+// memory fits too.  FP64: 192 threads (255 registers).
 #ifndef CLV_TILE_MAX_THREADS
 #define CLV_TILE_MAX_THREADS 384
 #endif
+constexpr int kTileThreadsF64 = CLV_TILE_MAX_THREADS < 192 ? CLV_TILE_MAX_THREADS : 192;
 template <typename R> struct TileBound {
-  static constexpr int threads = sizeof(R) == 4 ? CLV_TILE_MAX_THREADS : (CLV_TILE_MAX_THREADS < 128 ? CLV_TILE_MAX_THREADS : 128);
+  static constexpr int threads = sizeof(R) == 4 ? CLV_TILE_MAX_THREADS : kTileThreadsF64;
 };
 
 // One tile-chunk (index bidx within its event) of a stage; every thread of
