@@ -292,9 +292,9 @@ clv_status clv_mlp_train(float* d_params, float* d_work, const float* d_X, const
  * (CLV_EINVAL).  The batch starts (first-step predictor) at the first
  * clv_step, after every event's initial state was set.
  * Each event's tile follows a tiling policy shared by the batch: at most
- * max_threads threads per CTA (TJ as large as that allows, TK from neta, at
- * most 32 columns) and x chunks of about `chunk` planes; the default is 384
- * (128 in FP64) threads and 32 planes.  The persistent stage launch holds as
+ * max_threads threads per CTA (the shape with the least modelled cost) and x
+ * chunks of about `chunk` planes; the default is 384 (128 in FP64) threads and
+ * the chunk whose work items end soonest in the model.  The persistent stage launch holds as
  * many CTAs per SM as the device's occupancy calculator allows for the
  * policy's largest tile.  clv_autotune on a started batch
  * times the current policy and up to max_candidates others (thread caps of

@@ -9,6 +9,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <functional>
 #include <string>
 #include <vector>
 
@@ -1827,25 +1828,75 @@ clv_status clv_autotune(clv_handle* h, int max_candidates, int reps, clv_tile_in
 // ---------------- batch of events ----------------
 }  // extern "C"
 
-// Tile of one event of a batch under a tiling policy: TK from the eta_s
-// extent (at most 32 columns), TJ as large as the thread cap allows (at most
-// maxthr threads per CTA), x chunks of about `chunk` planes.
+// Tile of one event of a batch under a tiling policy: of the shapes of at most
+// maxthr threads per CTA (eta_s in 1..4 columns of tiles or columns of at most
+// 32, y tiles from the largest down to a third of it) the one whose tiles cost
+// a plane of the event least (plane_cost), x chunks of about `chunk` planes.
 static TileArgs batch_tile(const clv_config& c, int maxthr_cap, int chunk) {
   TileArgs t;
   const int maxthr = std::min(tile_max_threads(&c), maxthr_cap);
-  const int nk = (c.neta + 31) / 32;
-  t.TK = (c.neta + nk - 1) / nk;
-  t.TJ = std::max(1, std::min(c.ny, maxthr / (t.TK + 1) - 1));
   const size_t rsize = c.precision == CLV_FP64 ? 8 : 4;
-  auto smem_of = [&](int TJ) {
-    return c.eta_over_s > 0 ? tile_smem_bytes<true>(TJ, t.TK, rsize) : tile_smem_bytes<false>(TJ, t.TK, rsize);
-  };
-  while (t.TJ > 1 && smem_of(t.TJ) > kSmemOptinMax) --t.TJ;
+  double best = 1e300;
+  t.TJ = t.TK = 1;
+  const int columns = std::max(4, (c.neta + 31) / 32);
+  for (int nk = 1; nk <= c.neta && (nk <= columns || best == 1e300); ++nk) {   // on to narrow tiles under a low cap
+    const int TK = (c.neta + nk - 1) / nk;
+    const int most = std::min(c.ny, maxthr / (TK + 1) - 1);
+    for (int TJ = most; TJ >= std::max(1, most / 3); --TJ) {
+      const size_t sm = c.eta_over_s > 0 ? tile_smem_bytes<true>(TJ, TK, rsize) : tile_smem_bytes<false>(TJ, TK, rsize);
+      if (sm > kSmemOptinMax) continue;
+      const double cost = (double)((c.ny + TJ - 1) / TJ) * ((c.neta + TK - 1) / TK) * plane_cost(&c, TJ, TK, 1);
+      if (cost < best) { best = cost; t.TJ = TJ; t.TK = TK; }
+    }
+  }
   const int nch = (c.nx + chunk - 1) / chunk;
   t.CX = (c.nx + nch - 1) / nch;
   t.ntj = (c.ny + t.TJ - 1) / t.TJ;
   t.ntk = (c.neta + t.TK - 1) / t.TK;
   return t;
+}
+
+// Work items (event, tile-chunk) of a batch under a policy with their modelled
+// costs, most expensive first.
+static std::vector<std::pair<double, int2>> batch_work(const clv_handle* h, int maxthr, int chunk,
+                                                       std::vector<TileArgs>& tiles) {
+  std::vector<std::pair<double, int2>> items;
+  tiles.clear();
+  for (size_t e = 0; e < h->batch.size(); ++e) {
+    const auto& ev = h->batch[e];
+    const TileArgs t = batch_tile(ev.cfg, maxthr, chunk);
+    tiles.push_back(t);
+    const int per = t.ntj * t.ntk, nb = per * ((ev.cfg.nx + t.CX - 1) / t.CX);
+    const double plane = plane_cost(&ev.cfg, t.TJ, t.TK, 1) * (ev.viscous ? 1.0 : 0.5);
+    for (int b = 0; b < nb; ++b) {
+      const int planes = std::min(t.CX, ev.cfg.nx - b / per * t.CX);
+      items.push_back({(planes + halo_planes(&ev.cfg)) * plane, make_int2((int)e, b)});
+    }
+  }
+  std::stable_sort(items.begin(), items.end(), [](const auto& a, const auto& b) { return a.first > b.first; });
+  return items;
+}
+
+// x chunk of the default policy: the one whose items, taken in order by the
+// first idle of `slots` CTAs, are done soonest in the model (shorter chunks
+// even out the end of a stage, longer ones stage fewer halo planes).
+static int batch_default_chunk(const clv_handle* h, int maxthr, int slots) {
+  int best = 32;
+  double best_t = 1e300;
+  std::vector<TileArgs> tiles;
+  for (int chunk : {8, 12, 16, 20, 24, 32, 40, 48, 64, 96, 128}) {
+    const auto items = batch_work(h, maxthr, chunk, tiles);
+    std::vector<double> busy((size_t)slots, 0.0);   // min-heap of the CTAs' finishing times
+    double end = 0.0;
+    for (const auto& it : items) {
+      std::pop_heap(busy.begin(), busy.end(), std::greater<double>());
+      busy.back() += it.first;
+      end = std::max(end, busy.back());
+      std::push_heap(busy.begin(), busy.end(), std::greater<double>());
+    }
+    if (end < best_t) { best_t = end; best = chunk; }
+  }
+  return best;
 }
 
 template <typename R> static cudaError_t batch_upload(clv_handle* h) {
@@ -1885,28 +1936,18 @@ template <typename R> static cudaError_t batch_attributes(size_t smem) {
 static cudaError_t batch_schedule(clv_handle* h, int maxthr, int chunk, int sms, size_t smem_max) {
   maxthr = std::min(maxthr, h->rsize == 8 ? std::min(CLV_TILE_MAX_THREADS, kBlock / 2) : CLV_TILE_MAX_THREADS);
   const size_t ne = h->batch.size();
-  std::vector<TileArgs> tiles(ne);
-  std::vector<std::pair<double, int2>> items;
+  std::vector<TileArgs> tiles;
+  const std::vector<std::pair<double, int2>> items = batch_work(h, maxthr, chunk, tiles);
   size_t smem = 0;
   int thr = 0;
   for (size_t e = 0; e < ne; ++e) {
-    const auto& ev = h->batch[e];
-    const TileArgs t = batch_tile(ev.cfg, maxthr, chunk);
-    tiles[e] = t;
-    const size_t sm = ev.viscous ? tile_smem_bytes<true>(t.TJ, t.TK, h->rsize) : tile_smem_bytes<false>(t.TJ, t.TK, h->rsize);
+    const TileArgs& t = tiles[e];
+    const size_t sm =
+        h->batch[e].viscous ? tile_smem_bytes<true>(t.TJ, t.TK, h->rsize) : tile_smem_bytes<false>(t.TJ, t.TK, h->rsize);
     smem = std::max(smem, sm);
     thr = std::max(thr, (t.TJ + 1) * (t.TK + 1));
-    const int nch = (ev.cfg.nx + t.CX - 1) / t.CX;
-    const int nb = t.ntj * t.ntk * nch;
-    for (int b = 0; b < nb; ++b) {
-      const int ch = b / (t.ntj * t.ntk);
-      const int planes = std::min(t.CX, ev.cfg.nx - ch * t.CX);
-      const double cost = (planes + 4.0) * (t.TJ + 4.0) * (t.TK + 4.0) * (ev.viscous ? 2.0 : 1.0);
-      items.push_back({cost, make_int2((int)e, b)});
-    }
   }
   if (smem > smem_max) return cudaErrorInvalidValue;
-  std::stable_sort(items.begin(), items.end(), [](const auto& a, const auto& b) { return a.first > b.first; });
   std::vector<int2> it(items.size());
   for (size_t i = 0; i < items.size(); ++i) it[i] = items[i].second;
   cudaError_t err = cudaStreamSynchronize(h->stream);   // no launch of the old schedule is in flight
@@ -1988,9 +2029,9 @@ clv_status clv_create_batch(const clv_config* cfgs, int nevents, void* cuda_stre
     ev.viscous = ev.cfg.eta_over_s > 0.0;
     off += ev.N;
   }
-  // default policy: the largest tiles the thread limit allows, x chunks of about 32 planes
+  // default policy: tiles up to the thread limit, the chunk with the shortest modelled stage
   cudaError_t err = h->rsize == 8 ? batch_upload<double>(h) : batch_upload<float>(h);
-  if (err == cudaSuccess) err = batch_schedule(h, CLV_TILE_MAX_THREADS, 32, sms, smem_max);
+  if (err == cudaSuccess) err = batch_schedule(h, CLV_TILE_MAX_THREADS, batch_default_chunk(h, h->rsize == 8 ? kBlock / 2 : CLV_TILE_MAX_THREADS, sms), sms, smem_max);
   if (err == cudaSuccess) err = cudaMalloc((void**)&h->batch_ctr, 2 * sizeof(int));
   if (err != cudaSuccess) {
     clv_destroy(h);
