@@ -41,7 +41,7 @@ struct FoArgs {
   int cy, ce;              // hypercubes along y and eta: ny - 1, neta - 1
   long long ncube;
   R ef;
-  R h[4];                  // tau1 - tau0, dx, dy, deta
+  R h[4], ih[4];           // tau1 - tau0, dx, dy, deta and their inverses
   R x0[4];                 // tau0 and the coordinates of cell (0, 0, 0)
   R cof[4];                // h0 h1 h2 h3 / h_mu: the 3-volume covector of local edges -> physical
   int cartesian;
@@ -136,21 +136,15 @@ __global__ void __launch_bounds__(kThreads) fo_compact_kernel(const unsigned cha
   if (f) list[offsets[blockIdx.x] + before + __popc(b & ((1u << lane) - 1u))] = (int)c;
 }
 
-// value of a 5-array at a runtime index, by selects (no local memory)
-template <typename T>
-__device__ __forceinline__ T sel5(const T (&x)[5], int m) {
-  return m == 0 ? x[0] : m == 1 ? x[1] : m == 2 ? x[2] : m == 3 ? x[3] : x[4];
-}
-
 // level-set point on the simplex edge from inside vertex vi (value fi >= 0)
 // to outside vertex vo (fo < 0), in local coordinates of the hypercube
 template <typename R>
 __device__ __forceinline__ void edge_point(int vi, int vo, R fi, R fo, R p[4]) {
-  const R t = fi / (fi - fo);
+  const R t = fi / (fi - fo), back = R(1) - t;
 #pragma unroll
-  for (int ax = 0; ax < 4; ++ax) {
-    const R bi = (R)(vi >> ax & 1), bo = (R)(vo >> ax & 1);
-    p[ax] = bi + t * (bo - bi);
+  for (int ax = 0; ax < 4; ++ax) {   // bi + t (bo - bi) for bits bi, bo of the corners
+    const R to1 = vi >> ax & 1 ? R(1) : t, to0 = vi >> ax & 1 ? back : R(0);
+    p[ax] = vo >> ax & 1 ? to1 : to0;
   }
 }
 
@@ -195,11 +189,16 @@ __device__ __forceinline__ void add_tet(const FoArgs<R>& a, const R* p0, const R
   pc.A += A;
 }
 
-// the piece of the level set in the simplex with vertex corners v[5] and
-// values f[5] (f = eps - eps_f)
+// the piece of the level set in the simplex with vertex corners v[5] (also
+// packed, 4 bits each) and values f[5] (f = eps - eps_f); fs: the lane's five
+// values again in shared memory (stride 32), for access by a runtime index.
+// A piece is one tetrahedron (one vertex against four) or a prism of three
+// (two against three): tetrahedron m of either is points (m, m+1, m+2, m+3) of
+// a list of six, so that a warp with both kinds runs the points and the
+// tetrahedra once.
 template <typename R>
-__device__ void simplex_piece(const FoArgs<R>& a, const int (&v)[5], const R (&f)[5], const int (&perm)[4],
-                              Piece<R>& pc) {
+__device__ __forceinline__ void simplex_piece(const FoArgs<R>& a, unsigned vpack, const R (&f)[5], const int (&perm)[4],
+                                              const R* fs, Piece<R>& pc) {
   unsigned inmask = 0;
 #pragma unroll
   for (int m = 0; m < 5; ++m) inmask |= (f[m] >= R(0) ? 1u : 0u) << m;
@@ -212,54 +211,44 @@ __device__ void simplex_piece(const FoArgs<R>& a, const int (&v)[5], const R (&f
 #pragma unroll
     for (int m = 0; m < 4; ++m)
       if (perm[m] == ax) d = f[m + 1] - f[m];
-    grad[ax] = d / a.h[ax];
+    grad[ax] = d * a.ih[ax];
   }
   const R gn = sqrt(grad[0] * grad[0] + grad[1] * grad[1] + grad[2] * grad[2] + grad[3] * grad[3]);
   if (!(gn > R(0))) return;  // only when the differences underflow: no piece
+  const R ign = R(1) / gn;
   R nhat[4];
 #pragma unroll
-  for (int ax = 0; ax < 4; ++ax) nhat[ax] = -grad[ax] / gn;
+  for (int ax = 0; ax < 4; ++ax) nhat[ax] = -grad[ax] * ign;
   // minority side (one or two vertices) against the majority, each in
-  // increasing vertex order
+  // increasing vertex order, as lists of 4-bit vertex numbers
   const bool min_in = nin <= 2;
   unsigned mm = min_in ? inmask : (~inmask & 31u);
   unsigned MM = ~mm & 31u;
-  int mi[2], Mi[4];
-#pragma unroll
-  for (int r = 0; r < 2; ++r) {
-    mi[r] = mm ? __ffs(mm) - 1 : 0;
-    mm &= mm - 1u;
-  }
+  const int nmin = __popc(mm);
+  const unsigned m0 = __ffs(mm) - 1, m1 = nmin == 2 ? 31 - __clz(mm) : m0;
+  unsigned Ml = 0;
 #pragma unroll
   for (int s = 0; s < 4; ++s) {
-    Mi[s] = MM ? __ffs(MM) - 1 : 0;
+    Ml |= (MM ? __ffs(MM) - 1u : 0u) << (4 * s);
     MM &= MM - 1u;
   }
-  const int nmin = min_in ? nin : 5 - nin;
-  auto point = [&](int r, int s, R p[4]) {
-    const int vm = mi[r], vM = Mi[s];
-    if (min_in) edge_point<R>(sel5(v, vm), sel5(v, vM), sel5(f, vm), sel5(f, vM), p);
-    else edge_point<R>(sel5(v, vM), sel5(v, vm), sel5(f, vM), sel5(f, vm), p);
+  // point of the edge from minority vertex vm to majority vertex vM
+  auto point = [&](unsigned vm, unsigned vM, R p[4]) {
+    const unsigned vi = min_in ? vm : vM, vo = min_in ? vM : vm;
+    edge_point<R>(vpack >> (4 * vi) & 15u, vpack >> (4 * vo) & 15u, fs[32 * vi], fs[32 * vo], p);
   };
-  if (nmin == 1) {
-    R q0[4], q1[4], q2[4], q3[4];
-    point(0, 0, q0);
-    point(0, 1, q1);
-    point(0, 2, q2);
-    point(0, 3, q3);
-    add_tet<R>(a, q0, q1, q2, q3, nhat, pc);
-  } else {
-    // prism: triangles (0, s) and (1, s), lateral edges (0, s) - (1, s)
-    R q00[4], q01[4], q02[4], q10[4], q11[4], q12[4];
-    point(0, 0, q00);
-    point(0, 1, q01);
-    point(0, 2, q02);
-    point(1, 0, q10);
-    point(1, 1, q11);
-    point(1, 2, q12);
-    add_tet<R>(a, q00, q01, q02, q10, nhat, pc);
-    add_tet<R>(a, q01, q02, q10, q11, nhat, pc);
-    add_tet<R>(a, q02, q10, q11, q12, nhat, pc);
+  // (0, 0) (0, 1) (0, 2), then (0, 3) of a tetrahedron or (1, 0) (1, 1) (1, 2) of a prism
+  R q[4][4];
+  point(m0, Ml & 15u, q[0]);
+  point(m0, Ml >> 4 & 15u, q[1]);
+  point(m0, Ml >> 8 & 15u, q[2]);
+  point(m1, nmin == 1 ? Ml >> 12 & 15u : Ml & 15u, q[3]);
+  add_tet<R>(a, q[0], q[1], q[2], q[3], nhat, pc);
+  if (nmin == 2) {
+    point(m1, Ml >> 4 & 15u, q[0]);
+    add_tet<R>(a, q[1], q[2], q[3], q[0], nhat, pc);
+    point(m1, Ml >> 8 & 15u, q[1]);
+    add_tet<R>(a, q[2], q[3], q[0], q[1], nhat, pc);
   }
 }
 
@@ -274,7 +263,7 @@ __device__ __forceinline__ R warp_sum(R x) {
 // the warps are latency-bound, and 32 resident warps per SM instead of 24
 // (78 registers) made a find 5% faster.
 template <typename R>
-__global__ void __launch_bounds__(kElemThreads, 4) fo_elements_kernel(FoArgs<R> a, const int* __restrict__ list,
+__global__ void __launch_bounds__(kElemThreads, sizeof(R) == 4 ? 4 : 2) fo_elements_kernel(FoArgs<R> a, const int* __restrict__ list,
                                                                    const long long* __restrict__ total,
                                                                    long long capacity, R* __restrict__ rec,
                                                                    int64_t* __restrict__ cube_out) {
@@ -298,6 +287,11 @@ __global__ void __launch_bounds__(kElemThreads, 4) fo_elements_kernel(FoArgs<R> 
   v[0] = 0;
 #pragma unroll
   for (int m = 0; m < 4; ++m) v[m + 1] = v[m] | (1 << perm[m]);
+  unsigned vpack = 0;
+#pragma unroll
+  for (int m = 0; m < 5; ++m) vpack |= (unsigned)v[m] << (4 * m);
+  __shared__ R s_f[kElemThreads / 32][5][32];   // each lane's own values
+  R* fs = &s_f[threadIdx.x >> 5][0][lane];
 
   long long n = *total;
   if (n > capacity) n = capacity;
@@ -310,12 +304,15 @@ __global__ void __launch_bounds__(kElemThreads, 4) fo_elements_kernel(FoArgs<R> 
     if (lane < 16) fq = a.e[lane & 1][corner_offset(a, i, j, k, lane)] - a.ef;
     R f[5];
 #pragma unroll
-    for (int m = 0; m < 5; ++m) f[m] = __shfl_sync(kFull, fq, v[m]);
+    for (int m = 0; m < 5; ++m) {
+      f[m] = __shfl_sync(kFull, fq, v[m]);
+      fs[32 * m] = f[m];
+    }
     Piece<R> pc;
 #pragma unroll
     for (int m = 0; m < 4; ++m) pc.dS[m] = pc.Ac[m] = 0;
     pc.A = 0;
-    if (lane < 24) simplex_piece<R>(a, v, f, perm, pc);
+    if (lane < 24) simplex_piece<R>(a, vpack, f, perm, fs, pc);
     R dS[4], Ac[4];
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
@@ -465,6 +462,7 @@ clv_status fo_run(const clv_fo_grid* g, const clv_fo_slice* s0, const clv_fo_sli
   const double vol = h[0] * h[1] * h[2] * h[3];
   for (int m = 0; m < 4; ++m) {
     a.h[m] = (R)h[m];
+    a.ih[m] = (R)(1.0 / h[m]);
     a.x0[m] = (R)x0[m];
     a.cof[m] = (R)(vol / h[m]);
   }
