@@ -299,7 +299,8 @@ std::vector<TileGeom> tile_candidates(const clv_config* c, int sms, size_t smem_
       const int occ = tile_occupancy(c, g.threads, g.smem);
       const long long slots = (long long)sms * occ;
       const long long waves = ((long long)g.blocks + slots - 1) / slots;
-      v.push_back({(double)waves * (g.t.CX + halo_planes(c)) * plane_cost(c, TJ, TK, occ), g});
+      const int share = (int)std::min<long long>(occ, ((long long)g.blocks + sms - 1) / sms);   // CTAs that do share an SM
+      v.push_back({(double)waves * (g.t.CX + halo_planes(c)) * plane_cost(c, TJ, TK, share), g});
     }
   }
   std::stable_sort(v.begin(), v.end(), [](const auto& a, const auto& b) { return a.first < b.first; });
