@@ -456,8 +456,7 @@ StageParams<R> stage_params(clv_handle* h, int stage) {
   p.nep = h->nep;
   p.xhalo = c.halo_x > 0 ? 1 : 0;
   p.N = h->N;
-  p.tau_dev = &h->tau_dev[h->cur].tau;
-  p.itau = h->tau_dev[h->cur].itau;
+  p.tau_dev = h->tau_dev + h->cur;
   p.tau_next = s1 ? nullptr : h->tau_dev + h->prev;   // prev becomes cur after the step
   p.dtau_d = c.dtau;
   p.cartesian = c.cartesian;
@@ -468,7 +467,7 @@ StageParams<R> stage_params(clv_handle* h, int stage) {
   p.st_tau = (R)(c.cartesian ? 0.0 : 1.0);
   p.eps_cut = (R)c.eps_cut;
   p.eps_cut_d = c.eps_cut;
-  p.deta_d = c.deta;
+  p.inv_deta = 1.0 / c.deta;
   p.is = is_coef<R>(c);
   p.polish_E = (R)(1.01 * c.eps_cut);
   p.polish_v = (R)0.99;   // gamma above ~7: E/eps > ~65, the FP32 eps = E - M v loses digits
@@ -561,14 +560,14 @@ void launch_stage(clv_handle* h, const StageParams<R>& p, bool timed) {
   if (timed) timing_event(h);
 }
 
-__global__ void set_tau_kernel(TauSlot* s, double tau, double dtau, int cartesian) {
-  store_tau(s, tau, dtau, cartesian);
+__global__ void set_tau_kernel(TauSlot* s, double tau, double dtau, double inv_deta, int cartesian) {
+  store_tau(s, tau, 1.0 / tau, dtau, inv_deta, cartesian);
 }
 
 // tau of the next step (from the primitive set cur)
 void set_tau(clv_handle* h, double tau) {
   h->tau = tau;
-  set_tau_kernel<<<1, 1, 0, h->stream>>>(h->tau_dev + h->cur, tau, h->cfg.dtau, h->cfg.cartesian);
+  set_tau_kernel<<<1, 1, 0, h->stream>>>(h->tau_dev + h->cur, tau, h->cfg.dtau, 1.0 / h->cfg.deta, h->cfg.cartesian);
 }
 
 // Half of a Heun step: stage 1, or stage 2 with the end-of-step bookkeeping
@@ -1907,7 +1906,7 @@ template <typename R> static cudaError_t batch_upload(clv_handle* h) {
   for (size_t e = 0; e < ne; ++e) {
     const auto& ev = h->batch[e];
     const clv_config& c = ev.cfg;
-    g[e] = EventGeom<R>{ev.off, c.nx, c.ny, c.neta, ev.nep, (R)(1.0 / c.dx), (R)(1.0 / c.dy), is_coef<R>(c), c.deta,
+    g[e] = EventGeom<R>{ev.off, c.nx, c.ny, c.neta, ev.nep, (R)(1.0 / c.dx), (R)(1.0 / c.dy), is_coef<R>(c), 1.0 / c.deta,
                         ev.viscous ? 1 : 0};
     t[e] = ev.tile;
   }

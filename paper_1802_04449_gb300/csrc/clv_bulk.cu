@@ -72,8 +72,8 @@ __global__ void __launch_bounds__(kBlock) bulk_stage_kernel(const StageParams<R>
   if (k >= p.ne) return;   // padding slot of the eta pitch
   const long long row = c / p.nep;
   const int j = (int)(row % p.ny), i = (int)(row / p.ny);
-  const TauS<R> ts = tau_scalars(p, STAGE);
-  const R inv_dl[3] = {p.inv_dl[0], p.inv_dl[1], (R)(1.0 / (ts.taus_d * p.deta_d))};
+  const TauFactors<R> ts = tau_factors(p, STAGE);
+  const R inv_dl[3] = {p.inv_dl[0], p.inv_dl[1], ts.inv_de};
   R S = R(0), div = R(0);
 #pragma unroll
   for (int ax = 0; ax < 3; ++ax) {

@@ -39,20 +39,45 @@ template <typename R> struct IsCoef {
 // sources stay FP32); the update adds the FP32 increment to the pair exactly,
 // and the recovery forms E and M from the pair.  The FP64 path stores T~ in
 // T and leaves Tl unused.
-// tau of a step and 1/tau of its end (tau + dtau; 1 in Cartesian mode) as a
-// float-float pair for the FP32 recovery.  A handle has two, used by alternate
-// steps like the primitive sets: the last kernel of a step writes the next
-// one's while its own is still being read.
+// tau of a step and what its kernels take from it: 1/tau of its end (tau +
+// dtau; 1 in Cartesian mode) as a float-float pair for the FP32 recovery, and
+// per stage the tau factors of TauS in both precisions.  One thread forms them
+// per step: formed by every thread of a kernel, their FP64 divisions alone took
+// the FP64 pipe (2 lanes an SM and cycle) 18 us on 97 x 97 x 41 cells and 2 us
+// of every CTA of a stage.  A handle has two slots, used by alternate steps
+// like the primitive sets: the last kernel of a step writes the next one's
+// while its own is still being read.
+template <typename R> struct TauFactors {
+  R taus, geo, inv_de;   // tau_s, 1/tau_s (Milne) or 0 (Cartesian), 1/(tau_s deta)
+};
 struct TauSlot {
   double tau;
   float itau[2];
+  double inv_taus[2];           // 1/tau_s of stages 1 and 2 (Cartesian: 1)
+  TauFactors<double> d[2];
+  TauFactors<float> f[2];
+  double taus_new;              // tau scale at the end of the step
+  double inv_end;               // 1/(tau + dtau)
 };
-__device__ __forceinline__ void store_tau(TauSlot* s, double tau, double dtau, int cartesian) {
-  const double x = cartesian ? 1.0 : 1.0 / (tau + dtau);
+// it: 1/tau
+__device__ __forceinline__ void store_tau(TauSlot* s, double tau, double it, double dtau, double inv_deta,
+                                          int cartesian) {
+  const double end = tau + dtau, ie = 1.0 / end;
+  const double x = cartesian ? 1.0 : ie;
   const float hi = (float)x;
   s->tau = tau;
   s->itau[0] = hi;
   s->itau[1] = (float)(x - (double)hi);
+  s->taus_new = cartesian ? 1.0 : end;
+  s->inv_end = ie;
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const double taus = cartesian ? 1.0 : k ? end : tau, inv = cartesian ? 1.0 : k ? ie : it;
+    const double geo = cartesian ? 0.0 : inv, inv_de = inv * inv_deta;
+    s->inv_taus[k] = inv;
+    s->d[k] = TauFactors<double>{taus, geo, inv_de};
+    s->f[k] = TauFactors<float>{(float)taus, (float)geo, (float)inv_de};
+  }
 }
 
 template <typename R> struct StageParams {
@@ -79,9 +104,8 @@ template <typename R> struct StageParams {
   long long N;
   // tau of the step lives on the device (advanced by a kernel after every
   // step), so the launches of a step do not depend on it and a captured step
-  // replays unchanged; tau_scalars() forms the stage's tau factors from it
-  const double* tau_dev;
-  const float* itau;   // FP32 path: 1/tau at the end of the step (Cartesian: 1) as a float-float pair
+  // replays unchanged
+  const TauSlot* tau_dev;
   TauSlot* tau_next;   // stage 2: tau of the next step, written by the root solve (nullptr in stage 1)
   double dtau_d;
   int cartesian;
@@ -93,7 +117,7 @@ template <typename R> struct StageParams {
   IsCoef<R> is;       // Israel-Stewart coefficients (tau_pi, lambda_1)
   R polish_E, polish_v;   // FP32: FP64 Newton where the FP32 eps < polish_E or M > polish_v E
   double eps_cut_d;
-  double deta_d;   // d eta_s in FP64 (1/(tau deta) is formed in the kernels, per event in a batch)
+  double inv_deta; // 1/d eta_s in FP64
   // reductions and error reporting
   double* block_sum;             // per block: sum of new T~^{tau tau} (stats launches only)
   unsigned long long* emax_bits; // max eps as the bits of a non-negative double
@@ -162,30 +186,16 @@ template <> struct SolveTraits<double> {
   static constexpr int maxit = 100;
 };
 
-// Reconstructed interface quantities (KT, Eq. flux_out): T~^{tau mu} (4),
-// pi~ (10), u~^tau, v^a = u~^a/u~^tau, P.
-// The tau factors of a stage, rounded to R exactly as a host computation in
-// FP64 would be: tau_s = tau at the stage (stage 1: tau_n, stage 2:
-// tau_n + dtau), or 1 in Cartesian coordinates.
-template <typename R> struct TauS {
-  double taus_d;   // tau_s in FP64
-  R taus;          // tau_s
-  R geo;           // 1/tau_s (Milne) or 0 (Cartesian)
-  R taus_new;      // tau scale at the end of the step (primitive recovery)
-};
+// The tau factors of a stage: tau_s = tau at the stage (stage 1: tau_n, stage
+// 2: tau_n + dtau), or 1 in Cartesian coordinates.
 template <typename R>
-__device__ __forceinline__ TauS<R> tau_scalars(const StageParams<R>& p, int stage) {
-  const double tn = *p.tau_dev;
-  const double tn1 = tn + p.dtau_d;
-  const double tst = stage == 1 ? tn : tn1;
-  TauS<R> t;
-  t.taus_d = p.cartesian ? 1.0 : tst;
-  t.taus = (R)t.taus_d;
-  t.geo = (R)(p.cartesian ? 0.0 : 1.0 / tst);
-  t.taus_new = (R)(p.cartesian ? 1.0 : tn1);
-  return t;
+__device__ __forceinline__ TauFactors<R> tau_factors(const StageParams<R>& p, int stage) {
+  if constexpr (sizeof(R) == 4) return p.tau_dev->f[stage - 1];
+  else return p.tau_dev->d[stage - 1];
 }
 
+// Reconstructed interface quantities (KT, Eq. flux_out): T~^{tau mu} (4),
+// pi~ (10), u~^tau, v^a = u~^a/u~^tau, P.
 template <bool VISC> struct NRec { static constexpr int n = VISC ? 17 : 7; };
 
 template <typename R, bool VISC>
@@ -280,7 +290,7 @@ __device__ __forceinline__ IdealPart<R, VISC> ideal_part(const StageParams<R>& p
                                                         const R pi4[4], R tn) {
   IdealPart<R, VISC> a;
   if constexpr (sizeof(R) == 4) {
-    const ff itn{p.itau[0], p.itau[1]};
+    const ff itn{p.tau_dev->itau[0], p.tau_dev->itau[1]};
     a.E = ff_mul(ff{Tv[0], Tlv[0]}, itn);
     if constexpr (VISC) a.E = ff_add(a.E, -pi4[0]);
 #pragma unroll
@@ -457,9 +467,9 @@ __global__ void __launch_bounds__(kBlock) stage_kernel(const StageParams<R> p) {
     constexpr int NR = NRec<VISC>::n;
     constexpr int NQ = VISC ? 14 : 4;
     constexpr int IU = VISC ? 14 : 4, IV = IU + 1;
-    const TauS<R> ts = tau_scalars(p, STAGE);
+    const TauFactors<R> ts = tau_factors(p, STAGE);
     const R taus = ts.taus;
-    const R inv_dl[3] = {p.inv_dl[0], p.inv_dl[1], (R)(1.0 / (ts.taus_d * p.deta_d))};
+    const R inv_dl[3] = {p.inv_dl[0], p.inv_dl[1], ts.inv_de};
     R S[NQ];
 #pragma unroll
     for (int q = 0; q < NQ; ++q) S[q] = R(0);
@@ -626,7 +636,7 @@ __global__ void __launch_bounds__(kBlock) stage_kernel(const StageParams<R> p) {
 #pragma unroll
       for (int m = 0; m < 4; ++m) pi4[m] = pinew[m];
     }
-    const IdealPart<R, VISC> ip = ideal_part<R, VISC>(p, Tnew, Tnl, pi4, tau_scalars(p, 1).taus_new);
+    const IdealPart<R, VISC> ip = ideal_part<R, VISC>(p, Tnew, Tnl, pi4, (R)p.tau_dev->taus_new);
     const R E = ip.e, Mx = ip.m[0], My = ip.m[1], Me = ip.m[2];
     R en = R(0), ux = R(0), uy = R(0), ue = R(0);
     R Pb = p.Pib ? p.Pib[c] : R(0);   // bulk pressure of the stage's output
@@ -684,7 +694,7 @@ __global__ void __launch_bounds__(kBlock) stage_kernel(const StageParams<R> p) {
     my_T0 = (double)Tnew[0] + (sizeof(R) == 4 ? (double)Tnl[0] : 0.0);
     my_e = (double)en;
   }
-  if (STAGE == 2 && c == 0) store_tau(p.tau_next, *p.tau_dev + p.dtau_d, p.dtau_d, p.cartesian);
+  if (STAGE == 2 && c == 0) store_tau(p.tau_next, p.tau_dev->tau + p.dtau_d, p.tau_dev->inv_end, p.dtau_d, p.inv_deta, p.cartesian);
   // ---------------- counters and reductions ----------------
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
@@ -741,7 +751,7 @@ __global__ void __launch_bounds__(kBlock, RecoverMinBlocks<R>::value) recover_ke
   double my_T0 = 0.0, my_e = 0.0;
   int my_iters = 0, my_solved = 0, my_polish_iters = 0;
   bool f_rescaled = false, f_fail = false, f_polished = false, f_nonfinite = false, f_nonconv = false;
-  const R tn = tau_scalars(p, 1).taus_new;
+  const R tn = (R)p.tau_dev->taus_new;
   // the ideal part E, M of the new T~ (FP32 path: unrounded float-floats for
   // the correction step, their high parts for the FP32 solve)
   double T0v = 0.0;
@@ -896,7 +906,7 @@ __global__ void __launch_bounds__(kBlock, RecoverMinBlocks<R>::value) recover_ke
     my_T0 = T0v;
     my_e = (double)en;
   }
-  if (p.tau_next && c == 0) store_tau(p.tau_next, *p.tau_dev + p.dtau_d, p.dtau_d, p.cartesian);
+  if (p.tau_next && c == 0) store_tau(p.tau_next, p.tau_dev->tau + p.dtau_d, p.tau_dev->inv_end, p.dtau_d, p.inv_deta, p.cartesian);
   const unsigned full = 0xffffffffu;
   const unsigned b_res = __ballot_sync(full, f_rescaled);
   const unsigned b_fail = __ballot_sync(full, f_fail);

@@ -45,7 +45,7 @@ template <typename R> struct EventGeom {
   int nep;            // eta pitch (ne rounded up to a multiple of 4)
   R inv_dx, inv_dy;
   IsCoef<R> is;
-  double deta;
+  double inv_deta;
   int viscous;        // batch: 1 if the event has eta/s > 0
 };
 
@@ -219,7 +219,7 @@ template <typename R> struct TileBound {
 // One tile-chunk (index bidx within its event) of a stage; every thread of
 // the block calls it (threads beyond the tile's (TJ+1)(TK+1) only take part
 // in the barriers).
-template <typename R, int STAGE, bool VISC>
+template <typename R, int STAGE, bool VISC, bool BATCH>
 __device__ __forceinline__ void stage_tile_body(const StageParams<R>& p, const EventGeom<R>& ev, const TileArgs& t,
                                                 int bidx, unsigned char* smem_raw) {
   using L = Box<VISC>;
@@ -257,11 +257,11 @@ __device__ __forceinline__ void stage_tile_body(const StageParams<R>& p, const E
   const bool active = is_cell && j < ev.ny && k < ev.ne;
   const int cid = ta * t.TK + tb;                  // cell slot (valid when is_cell)
   const int center = (ta + 2) * BW + (tb + coff);  // box cell of (ta, tb)
-  const TauS<R> ts = tau_scalars(p, STAGE);
+  const TauFactors<R> ts = tau_factors(p, STAGE);
   const R taus = ts.taus;
   const R inv_dx = ev.inv_dx;
   const R inv_dy = ev.inv_dy;
-  const R inv_de = (R)(1.0 / (ts.taus_d * ev.deta));   // 1/(tau deta)
+  const R inv_de = BATCH ? (R)(p.tau_dev->inv_taus[STAGE - 1] * ev.inv_deta) : ts.inv_de;   // 1/(tau deta)
 
   R W0[NF], W1[NF];      // staged fields of the own column at planes pl-2, pl-1
   R S0[NR];              // x-slope at plane pl-2
@@ -570,8 +570,8 @@ __global__ void __launch_bounds__(TileBound<R>::threads, 1)
     stage_tile_kernel(const StageParams<R> p, const TileArgs t) {
   enter_step_kernel();
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const EventGeom<R> ev{0, p.nx, p.ny, p.ne, p.nep, p.inv_dl[0], p.inv_dl[1], p.is, p.deta_d, VISC ? 1 : 0};
-  stage_tile_body<R, STAGE, VISC>(p, ev, t, blockIdx.x, smem_raw);
+  const EventGeom<R> ev{0, p.nx, p.ny, p.ne, p.nep, p.inv_dl[0], p.inv_dl[1], p.is, p.inv_deta, VISC ? 1 : 0};
+  stage_tile_body<R, STAGE, VISC, false>(p, ev, t, blockIdx.x, smem_raw);
 }
 
 // A batch of events stored back to back: one persistent launch (a CTA per
@@ -595,8 +595,8 @@ __global__ void __launch_bounds__(TileBound<R>::threads, 1)
     const int2 w = items[it];
     const EventGeom<R> ev = evs[w.x];
     const TileArgs t = tiles[w.x];
-    if (ANY_VISC && ev.viscous) stage_tile_body<R, STAGE, true>(p, ev, t, w.y, smem_raw);
-    else stage_tile_body<R, STAGE, false>(p, ev, t, w.y, smem_raw);
+    if (ANY_VISC && ev.viscous) stage_tile_body<R, STAGE, true, true>(p, ev, t, w.y, smem_raw);
+    else stage_tile_body<R, STAGE, false, true>(p, ev, t, w.y, smem_raw);
   }
 }
 
