@@ -193,6 +193,7 @@ clv_status validate(const clv_config* c) {
 
 // shared memory a block may opt in to on sm_100 / sm_103 (227 KiB)
 constexpr size_t kSmemOptinMax = 232448;
+constexpr size_t kOneCtaSmem = 233472 / 2;   // with the 1 KB that a CTA costs, two do not fit an SM
 
 struct TileGeom {
   TileArgs t;
@@ -276,6 +277,11 @@ TileGeom tile_geometry_of(const clv_config* c, int sms, int TJ, int TK, int cx) 
   t.CX = cx;
   const long long nch = (c->nx + t.CX - 1) / t.CX;
   g.blocks = (unsigned)(tiles * nch);
+  // a grid of at most one CTA per SM asks for more than half of an SM's shared
+  // memory: placed early, beside a predecessor that drains, its CTAs would
+  // else double up on some SMs and leave others idle (33 x 33 x 9 in FP64, 132
+  // CTAs: 132 us a step instead of 99)
+  if (g.blocks <= (unsigned)sms) g.smem = std::max(g.smem, kOneCtaSmem);
   return g;
 }
 
@@ -299,8 +305,10 @@ std::vector<TileGeom> tile_candidates(const clv_config* c, int sms, size_t smem_
       const int occ = tile_occupancy(c, g.threads, g.smem);
       const long long slots = (long long)sms * occ;
       const long long waves = ((long long)g.blocks + slots - 1) / slots;
-      const int share = (int)std::min<long long>(occ, ((long long)g.blocks + sms - 1) / sms);   // CTAs that do share an SM
-      v.push_back({(double)waves * (g.t.CX + halo_planes(c)) * plane_cost(c, TJ, TK, share), g});
+      v.push_back({(double)waves * (g.t.CX + halo_planes(c)) * plane_cost(c, TJ, TK, occ), g});
+      if (occ == 1) continue;   // chunks for one CTA per SM as well
+      g = tile_geometry_of(c, sms, TJ, TK, chunk_planes(c->nx, (long long)g.t.ntj * g.t.ntk, sms, halo_planes(c)));
+      if (g.blocks <= (unsigned)sms) v.push_back({(g.t.CX + halo_planes(c)) * plane_cost(c, TJ, TK, 1), g});
     }
   }
   std::stable_sort(v.begin(), v.end(), [](const auto& a, const auto& b) { return a.first < b.first; });
