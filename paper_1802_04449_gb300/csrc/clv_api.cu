@@ -97,6 +97,7 @@ struct clv_handle {
   double tau = 0.0;               // host copy, advanced by the same additions
   long long step = 0;
   bool initialized = false;
+  bool initial_pi = false;   // the initial state came with pi~
   bool predictor_pending = false;   // x-slab: the first-step predictor is driven by clv_slab_predictor
   std::string last_error;
   // kernel timing (instrumentation)
@@ -429,6 +430,7 @@ template <typename R> EosView<R> eos_view(const clv_handle* h) {
   return v;
 }
 
+inline unsigned transfer_grid(long long n) { return (unsigned)((n + kBlock * kTransfer - 1) / (kBlock * kTransfer)); }
 inline unsigned grid_of(long long N) { return (unsigned)((N + kBlock - 1) / kBlock); }
 
 template <typename R> IsCoef<R> is_coef(const clv_config& c) {
@@ -594,6 +596,15 @@ void launch_half(clv_handle* h, int stage, bool stats, bool timed) {
     return;
   }
   StageParams<R> p2 = stage_params<R>(h, 2);
+  if (!VISC && h->viscous && h->batch.empty()) {
+    // the first-step predictor: only its velocities are wanted, so its T~ goes
+    // to the stage-2 shear buffers, which the first viscous stage overwrites,
+    // and the initial T~ stays
+    for (int m = 0; m < 4; ++m) {
+      p2.Tout[m] = (R*)h->PI1[m];
+      p2.Toutl[m] = (R*)h->PI1[4 + m];
+    }
+  }
   if (VISC && h->PB[0]) {   // bulk: Pi^{n+1} from Pi' and Pi^n, in place over Pi^n
     p2.Pib = (R*)h->PB[0];
     launch_bulk_stage<R>(p2, 2, h->PB[1], h->PB[0], h->PB[0], h->cfg.zeta_over_s, h->stream);
@@ -758,20 +769,24 @@ template <typename R> struct ConvertSet {
 };
 template <typename R>
 __global__ void __launch_bounds__(kBlock) convert_kernel(const ConvertSet<R> x, long long npad, int ne, int nep) {
-  const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= npad) return;
   const double* s = x.s[blockIdx.y];
-  long long row;
-  int k;
-  if (npad <= (1ll << 31)) {
-    const unsigned r = (unsigned)c / (unsigned)nep;
-    row = r;
-    k = (int)((unsigned)c - r * (unsigned)nep);
-  } else {
-    row = c / nep;
-    k = (int)(c - row * nep);
+  R* d = x.d[blockIdx.y];
+#pragma unroll
+  for (int i = 0; i < kTransfer; ++i) {
+    const long long c = ((long long)blockIdx.x * kTransfer + i) * kBlock + threadIdx.x;
+    if (c >= npad) return;
+    long long row;
+    int k;
+    if (npad <= (1ll << 31)) {
+      const unsigned r = (unsigned)c / (unsigned)nep;
+      row = r;
+      k = (int)((unsigned)c - r * (unsigned)nep);
+    } else {
+      row = c / nep;
+      k = (int)(c - row * nep);
+    }
+    d[c] = s && k < ne ? (R)s[row * ne + k] : R(0);
   }
-  x.d[blockIdx.y][c] = s && k < ne ? (R)s[row * ne + k] : R(0);
 }
 
 template <typename R> Prim<R> prim_at(Prim<R> p, long long off) {
@@ -808,9 +823,9 @@ clv_status load_initial_range(clv_handle* h, long long off, long long npad, long
       CLV_CUDA(h, cudaMemcpyAsync(h->staging, all.s[f], (size_t)nc * 8, cudaMemcpyHostToDevice, h->stream));
       one.s[0] = h->staging;
     }
-    convert_kernel<R><<<gp, kBlock, 0, h->stream>>>(one, npad, ne, nep);
+    convert_kernel<R><<<transfer_grid(npad), kBlock, 0, h->stream>>>(one, npad, ne, nep);
   }
-  if (!host) convert_kernel<R><<<dim3(gp, kMaxConvert), kBlock, 0, h->stream>>>(all, npad, ne, nep);
+  if (!host) convert_kernel<R><<<dim3(transfer_grid(npad), kMaxConvert), kBlock, 0, h->stream>>>(all, npad, ne, nep);
   init_primitives_kernel<R><<<gp, kBlock, 0, h->stream>>>(pc, pp, pi0, visc, eos_view<R>(h), c.eps_cut, npad);
   CLV_CUDA(h, cudaGetLastError());
   return CLV_OK;
@@ -851,7 +866,7 @@ template <typename R> clv_status initial_begin(clv_handle* h) {
 }
 
 // After the first-step predictor (one pi-free Heun step, Sec. 3): u~^{-1} =
-// 2 u~^0 - u~^1_ideal, tau and T~ (now with pi~) of the initial state again.
+// 2 u~^0 - u~^1_ideal, tau of the initial state again, and T~ now with pi~.
 template <typename R> clv_status initial_end(clv_handle* h) {
   const long long N = h->N;
   const unsigned g = grid_of(N);
@@ -862,9 +877,10 @@ template <typename R> clv_status initial_end(clv_handle* h) {
   extrapolate_prev_kernel<R><<<g, kBlock, 0, h->stream>>>(prim_set<R>(h, h->cur), prim_set<R>(h, h->prev), N);
   set_tau(h, c.tau0);
   h->step = 0;
-  tilde_T_kernel<R><<<g, kBlock, 0, h->stream>>>(prim_set<R>(h, h->cur), pi0, true, t_arrays<R>(h->T0),
-                                                 t_arrays<R>(h->TL0), h->TL0[0] != nullptr,
-                                                 c.cartesian ? 1.0 : c.tau0, N);
+  if (h->initial_pi || !h->batch.empty())   // else T~ is that of initial_begin still
+    tilde_T_kernel<R><<<g, kBlock, 0, h->stream>>>(prim_set<R>(h, h->cur), pi0, true, t_arrays<R>(h->T0),
+                                                   t_arrays<R>(h->TL0), h->TL0[0] != nullptr,
+                                                   c.cartesian ? 1.0 : c.tau0, N);
   CLV_CUDA(h, cudaMemsetAsync(h->dstats, 0, sizeof(DevStats), h->stream));
   CLV_CUDA(h, cudaGetLastError());
   h->predictor_pending = false;
@@ -895,6 +911,7 @@ template <typename R> clv_status finish_initial(clv_handle* h) {
 
 template <typename R>
 clv_status set_initial_impl(clv_handle* h, const double* const in[4], const double* pi, bool host) {
+  h->initial_pi = pi && h->viscous;
   clv_status s = load_initial_range<R>(h, 0, h->N, h->Nc, h->cfg.neta, h->nep, h->viscous, in, pi, host);
   return s != CLV_OK ? s : finish_initial<R>(h);
 }
@@ -931,7 +948,7 @@ clv_status export_fields(clv_handle* h, const int* which, int nf, double* dst, l
     field_source<R>(h, which[i], off, x.hi[m], x.lo[m]);
     x.dst[m++] = d;
   }
-  if (m) export_kernel<R><<<dim3(grid_of(n), (unsigned)m), kBlock, 0, h->stream>>>(x, n, ne, nep);
+  if (m) export_kernel<R><<<dim3(transfer_grid(n), (unsigned)m), kBlock, 0, h->stream>>>(x, n, ne, nep);
   CLV_CUDA(h, cudaGetLastError());
   return CLV_OK;
 }
@@ -1069,7 +1086,17 @@ __global__ void __launch_bounds__(kBlock) prims_from_T_kernel(double* a0, double
     atomicOr(err, 2u);
     e = ux = uy = ue = 0.0;
   } else {
-    const RootResult rr = solve_primitive<double, R, R>(eos, eps_cut, E, Mx, My, Me, 1e-15, 200, e, ux, uy, ue);
+    // single-precision handle: the FP64 solve starts from the FP32 root (two
+    // or three steps on the FP64 pipe instead of six)
+    double v0 = -1.0;
+    if constexpr (sizeof(R) == 4) {
+      float ef, a, b, d, vf = -1.0f;
+      solve_primitive<float, float>(eos, (float)eps_cut, (float)E, (float)Mx, (float)My, (float)Me,
+                                    SolveTraits<float>::tol, SolveTraits<float>::maxit, ef, a, b, d, &vf);
+      v0 = (double)vf;
+    }
+    const RootResult rr =
+        solve_primitive<double, R, R>(eos, eps_cut, E, Mx, My, Me, 1e-15, 200, e, ux, uy, ue, &v0);
     if (rr.rescaled) atomicAdd(counters + 0, 1ull);
     if (rr.iters < 0) { atomicAdd(counters + 1, 1ull); atomicOr(err, 1u); }
   }

@@ -748,7 +748,8 @@ __global__ void __launch_bounds__(kBlock, RecoverMinBlocks<R>::value) recover_ke
   const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const bool active = c < p.N;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-  double my_T0 = 0.0, my_e = 0.0;
+  double my_T0 = 0.0;
+  R my_e = R(0);
   int my_iters = 0, my_solved = 0, my_polish_iters = 0;
   bool f_rescaled = false, f_fail = false, f_polished = false, f_nonfinite = false, f_nonconv = false;
   const R tn = (R)p.tau_dev->taus_new;
@@ -904,7 +905,7 @@ __global__ void __launch_bounds__(kBlock, RecoverMinBlocks<R>::value) recover_ke
       }
     }
     my_T0 = T0v;
-    my_e = (double)en;
+    my_e = en;
   }
   if (p.tau_next && c == 0) store_tau(p.tau_next, p.tau_dev->tau + p.dtau_d, p.tau_dev->inv_end, p.dtau_d, p.inv_deta, p.cartesian);
   const unsigned full = 0xffffffffu;
@@ -944,8 +945,9 @@ __global__ void __launch_bounds__(kBlock, RecoverMinBlocks<R>::value) recover_ke
   }
   if constexpr (STATS) {
     __shared__ double s_sum[kBlock / 32];
-    __shared__ double s_max[kBlock / 32];
-    double sm = my_T0, mx = my_e;
+    __shared__ R s_max[kBlock / 32];
+    double sm = my_T0;
+    R mx = my_e;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       sm += __shfl_down_sync(full, sm, o);
@@ -954,10 +956,11 @@ __global__ void __launch_bounds__(kBlock, RecoverMinBlocks<R>::value) recover_ke
     if (lane == 0) { s_sum[wid] = sm; s_max[wid] = mx; }
     __syncthreads();
     if (threadIdx.x == 0) {
-      double a = 0.0, b = 0.0;
+      double a = 0.0;
+      R b = R(0);
       for (int w = 0; w < nwarp; ++w) { a += s_sum[w]; b = fmax(b, s_max[w]); }
       p.block_sum[blockIdx.x] = a;
-      if (b > 0.0) atomicMax(p.emax_bits, (unsigned long long)__double_as_longlong(b));
+      if (b > R(0)) atomicMax(p.emax_bits, (unsigned long long)__double_as_longlong((double)b));
     }
   }
 }
@@ -1127,15 +1130,35 @@ template <typename R> struct ExportSet {
   const R *hi[kMaxExport], *lo[kMaxExport];
   double* dst[kMaxExport];
 };
+// A normal float or a zero as a double by its bits: the FP64 pipe, which does
+// conversions, has 2 lanes an SM and cycle and would bound an export.
+__device__ __forceinline__ double widen(float x) {
+  const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
+  if (m - 0x00800000u < 0x7f000000u)
+    return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(b << 29));
+  if (m == 0) return __hiloint2double((int)b, 0);
+  return (double)x;
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+
+// Cells of a thread in the initial-state and export transfers: loads in flight
+// for the bandwidth.  Export of 18 fields of 261 x 261 x 121 cells: 0.80 ms
+// with one converted by the FP64 pipe.
+constexpr int kTransfer = 4;
+
 template <typename R>
 __global__ void __launch_bounds__(kBlock) export_kernel(const ExportSet<R> x, long long N, int ne, int nep) {
-  const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= N) return;
-  const long long k = padded_index(c, ne, nep);
   const R *hi = x.hi[blockIdx.y], *lo = x.lo[blockIdx.y];
-  double v = (double)hi[k];
-  if (lo) v += (double)lo[k];
-  x.dst[blockIdx.y][c] = v;
+  double* dst = x.dst[blockIdx.y];
+#pragma unroll
+  for (int i = 0; i < kTransfer; ++i) {
+    const long long c = ((long long)blockIdx.x * kTransfer + i) * kBlock + threadIdx.x;
+    if (c >= N) return;
+    const long long k = padded_index(c, ne, nep);
+    double v = widen(hi[k]);
+    if (lo) v += widen(lo[k]);
+    dst[c] = v;
+  }
 }
 
 // Deterministic final sum of the per-block partials (one block).
