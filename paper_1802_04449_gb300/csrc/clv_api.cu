@@ -326,7 +326,7 @@ TileGeom tile_geometry(const clv_config* c, int sms) {
   return v.empty() ? tile_geometry_of(c, sms, 1, 1, 0) : v.front();
 }
 
-constexpr int kRecoverSmall = 64;   // threads of a recovery block on a small grid (recover_block)
+constexpr int kRecoverSmall = 64;   // threads of the smaller recovery block (recover_block)
 
 inline int eta_pitch(int neta) { return (neta + 3) & ~3; }
 
@@ -528,10 +528,15 @@ template <typename R, bool VISC> cudaError_t tile_attributes(size_t smem) {
   return e;
 }
 
-// Threads of a recovery block: kBlock, or kRecoverSmall on a grid that would
-// not give every SM a block of kBlock (the cells of 33 x 33 x 9: 20 us with 52
-// blocks of 256 on 152 SMs in FP64, whose pipe is what the solve waits for).
-inline int recover_block(const clv_handle* h) { return (h->N + kBlock - 1) / kBlock < 2ll * h->sms ? kRecoverSmall : kBlock; }
+// Threads of a recovery block: kRecoverSmall, so that a block ends with its own
+// two warps' root solves (261 x 261 x 121 in FP32: stage 2 254 us with blocks
+// of 256, 235 with 64) and a small grid spreads over the SMs (33 x 33 x 9 in
+// FP64: 21 us with 52 blocks of 256, 14.5 with 64); kBlock with the network,
+// whose weights a block loads, on a grid that gives every SM two such blocks.
+inline int recover_block(const clv_handle* h) {
+  const bool net = h->rsize == 4 && (h->guess == kGuessMlp || h->guess == kGuessMlpAll);
+  return net && (h->N + kBlock - 1) / kBlock >= 2ll * h->sms ? kBlock : kRecoverSmall;
+}
 inline unsigned recover_grid(const clv_handle* h) {
   const int b = recover_block(h);
   return (unsigned)((h->N + b - 1) / b);
