@@ -220,7 +220,7 @@ int kernel_occupancy(const void* f, int threads, size_t smem) {
 // CTAs of a tile on one SM by its shared memory and registers (168 a thread in
 // FP32, 255 in FP64, as the launch bounds leave them)
 int tile_occupancy(const clv_config* c, int threads, size_t smem) {
-  const int warps = (threads + 31) / 32, regs = (c->precision == CLV_FP64 ? 256 : 168) * 32;
+  const int warps = (c->precision == CLV_FP64 ? kTileThreadsF64 : threads + 31) / 32, regs = (c->precision == CLV_FP64 ? 256 : 168) * 32;
   const int by_regs = 65536 / (warps * regs), by_smem = (int)(233472 / (smem + 1024));
   return std::max(1, std::min({by_regs, by_smem, 2048 / (32 * warps)}));
 }
@@ -229,13 +229,17 @@ int tile_occupancy(const clv_config* c, int threads, size_t smem) {
 // that a chunk costs beyond its own.  FP32: a plane is a chain of ~2000
 // dependent instructions whatever the tile, plus the box's cells (97 x 97 x 41
 // viscous stage 1: 7 x 22 tiles 4.8 us, 12 x 21 5.3, 16 x 21 6.0, two of 7 x 21
-// 5.8); the 4 halo planes, without y and eta interfaces, cost about 3.  FP64:
-// the cells and their halo on the FP64 pipe over a chain that is the longer
-// part of an ideal tile (33 x 33 x 9: 18 x 9 tiles 41 us, 9 x 9 35, 3 x 9 with
-// three planes 59; 97 x 97 x 41 viscous: 7 x 21 and 10 x 14 1.11 ms, 4 x 21
-// 1.35, 7 x 14 in two waves 1.24).
+// 5.8); the 4 halo planes, without y and eta interfaces, cost about 3.
+// FP64: warp passes of the busiest quarter of the SM (TileBound) times the FP64
+// instructions of an interface, of a cell with its x-interface and of a
+// conversion.
 double plane_cost(const clv_config* c, int TJ, int TK, int occ) {
-  if (c->precision == CLV_FP64) return (c->eta_over_s > 0.0 ? 200.0 : 435.0) + occ * (double)((TJ + 2) * (TK + 2));
+  if (c->precision == CLV_FP64) {
+    auto passes = [](int n) { return ((n + 31) / 32 + 3) / 4; };
+    const bool visc = c->eta_over_s > 0.0;
+    return (visc ? 110.0 : 65.0) * passes((TJ + 1) * TK + TJ * (TK + 1)) + (visc ? 240.0 : 130.0) * passes(TJ * TK) +
+           17.0 * passes(TJ * (TK + 4) + 4 * TK) + 30.0;
+  }
   return 620.0 + occ * (double)((TJ + 4) * box_width(TK));
 }
 inline double halo_planes(const clv_config* c) { return c->precision == CLV_FP64 ? 1.2 : 3.0; }
@@ -254,6 +258,11 @@ int chunk_planes(int nx, long long tiles, long long slots, double halo) {
     if (cost < best - 1e-9) { best = cost; best_nch = used; }
   }
   return (int)((nx + best_nch - 1) / best_nch);
+}
+
+// threads of a CTA whose tile has `positions` interface positions
+template <typename R> unsigned cta_threads(int positions) {
+  return (unsigned)(sizeof(R) == 8 ? kTileThreadsF64 : positions);
 }
 
 inline int tile_max_threads(const clv_config* c) {
@@ -558,8 +567,8 @@ template <typename R, bool VISC, int STAGE, bool STATS>
 void launch_stage(clv_handle* h, const StageParams<R>& p, bool timed) {
   if (!h->batch.empty()) {
     cudaMemsetAsync(h->batch_ctr + (STAGE - 1), 0, sizeof(int), h->stream);
-    launch_step_kernel(stage_batch_kernel<R, STAGE, VISC>, h->batch_blocks, h->batch_threads, h->batch_smem, h->stream,
-                       p, (const EventGeom<R>*)h->batch_geom, h->batch_tiles, h->batch_items, h->batch_nitems,
+    launch_step_kernel(stage_batch_kernel<R, STAGE, VISC>, h->batch_blocks, cta_threads<R>(h->batch_threads),
+                       h->batch_smem, h->stream, p, (const EventGeom<R>*)h->batch_geom, h->batch_tiles, h->batch_items, h->batch_nitems,
                        h->batch_ctr + (STAGE - 1));
     if (timed) timing_event(h);
     launch_recover<R, VISC, STATS>(h, p);
@@ -567,8 +576,8 @@ void launch_stage(clv_handle* h, const StageParams<R>& p, bool timed) {
     launch_step_kernel(stage_kernel<R, STAGE, VISC, STATS>, grid_of(h->N), kBlock, 0, h->stream, p);
     if (timed) timing_event(h);   // empty recovery slot
   } else {
-    launch_step_kernel(stage_tile_kernel<R, STAGE, VISC>, h->tile_blocks, h->tile_threads, h->tile_smem, h->stream, p,
-                       h->tile);
+    launch_step_kernel(stage_tile_kernel<R, STAGE, VISC>, h->tile_blocks, cta_threads<R>(h->tile_threads), h->tile_smem,
+                       h->stream, p, h->tile);
     if (timed) timing_event(h);
     launch_recover<R, VISC, STATS>(h, p);
   }
@@ -1488,7 +1497,7 @@ static cudaError_t time_stage1_batch(clv_handle* h, int reps, cudaEvent_t e0, cu
   const StageParams<R> p = stage_params<R>(h, 1);
   auto launch = [&]() {
     cudaMemsetAsync(h->batch_ctr, 0, sizeof(int), h->stream);
-    stage_batch_kernel<R, 1, VISC><<<h->batch_blocks, h->batch_threads, h->batch_smem, h->stream>>>(
+    stage_batch_kernel<R, 1, VISC><<<h->batch_blocks, cta_threads<R>(h->batch_threads), h->batch_smem, h->stream>>>(
         p, (const EventGeom<R>*)h->batch_geom, h->batch_tiles, h->batch_items, h->batch_nitems, h->batch_ctr);
   };
   launch();
@@ -1506,10 +1515,10 @@ static cudaError_t time_stage1_batch(clv_handle* h, int reps, cudaEvent_t e0, cu
 template <typename R, bool VISC>
 static cudaError_t time_stage1(clv_handle* h, int reps, cudaEvent_t e0, cudaEvent_t e1, double* ms) {
   const StageParams<R> p = stage_params<R>(h, 1);
-  stage_tile_kernel<R, 1, VISC><<<h->tile_blocks, h->tile_threads, h->tile_smem, h->stream>>>(p, h->tile);
+  stage_tile_kernel<R, 1, VISC><<<h->tile_blocks, cta_threads<R>(h->tile_threads), h->tile_smem, h->stream>>>(p, h->tile);
   cudaEventRecord(e0, h->stream);
   for (int r = 0; r < reps; ++r)
-    stage_tile_kernel<R, 1, VISC><<<h->tile_blocks, h->tile_threads, h->tile_smem, h->stream>>>(p, h->tile);
+    stage_tile_kernel<R, 1, VISC><<<h->tile_blocks, cta_threads<R>(h->tile_threads), h->tile_smem, h->stream>>>(p, h->tile);
   cudaEventRecord(e1, h->stream);
   cudaError_t e = cudaEventSynchronize(e1);
   if (e == cudaSuccess) e = cudaGetLastError();
@@ -2008,7 +2017,8 @@ static cudaError_t batch_schedule(clv_handle* h, int maxthr, int chunk, int sms,
   h->batch_threads = thr;
   h->batch_nitems = (int)it.size();
   const void* bk = h->rsize == 8 ? (const void*)stage_batch_kernel<double, 2, true> : (const void*)stage_batch_kernel<float, 2, true>;
-  h->batch_blocks = (unsigned)std::min<long long>((long long)sms * kernel_occupancy(bk, thr, smem), h->batch_nitems);
+  const int cta = (int)(h->rsize == 8 ? cta_threads<double>(thr) : cta_threads<float>(thr));
+  h->batch_blocks = (unsigned)std::min<long long>((long long)sms * kernel_occupancy(bk, cta, smem), h->batch_nitems);
   h->batch_maxthr = maxthr;
   h->batch_chunk = chunk;
   invalidate_graphs(h);   // captured steps hold the old launch shape and item list

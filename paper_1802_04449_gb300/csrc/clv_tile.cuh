@@ -204,21 +204,28 @@ __device__ __forceinline__ void box_interface(const R* box, int NB, int c, int s
   interface_flux<R, VISC>(Ls, Rs, cs[-stride], cs[0], ax, taus, H);
 }
 
-// Thread cap of a stage-kernel CTA.  FP32: 384 threads (12 warps) fit the
-// register file at the 168 registers that bound allows; a CTA of at most 192
-// threads then leaves room for a second one on the SM, when its shared
-// memory fits too.  FP64: 192 threads (255 registers).
+// Cap of a tile's (TJ+1)(TK+1) interface positions, and the bound of a CTA's
+// threads.  FP32: a thread per position, 384 (12 warps) fit the register file
+// at the 168 registers that bound allows; a CTA of at most 192 threads then
+// leaves room for a second one on the SM, when its shared memory fits too.
+// FP64: always 256 threads (8 warps of 255 registers).  A quarter of the SM
+// issues an FP64 warp instruction over 64 cycles whatever its active lanes, so
+// what a plane costs is the warp passes of the busiest quarter: the conversions
+// and the interfaces are spread over all warps as tasks and the cells over the
+// first threads, instead of a thread per position doing one of each (a 10 x 14
+// tile: six warps, two on two of the quarters, three of them converting four
+// cells in turn).
 #ifndef CLV_TILE_MAX_THREADS
 #define CLV_TILE_MAX_THREADS 384
 #endif
-constexpr int kTileThreadsF64 = CLV_TILE_MAX_THREADS < 192 ? CLV_TILE_MAX_THREADS : 192;
+constexpr int kTileThreadsF64 = 256;
 template <typename R> struct TileBound {
   static constexpr int threads = sizeof(R) == 4 ? CLV_TILE_MAX_THREADS : kTileThreadsF64;
 };
 
 // One tile-chunk (index bidx within its event) of a stage; every thread of
-// the block calls it (threads beyond the tile's (TJ+1)(TK+1) only take part
-// in the barriers).
+// the block calls it (FP32: threads beyond the tile's (TJ+1)(TK+1) only take
+// part in the barriers).
 template <typename R, int STAGE, bool VISC, bool BATCH>
 __device__ __forceinline__ void stage_tile_body(const StageParams<R>& p, const EventGeom<R>& ev, const TileArgs& t,
                                                 int bidx, unsigned char* smem_raw) {
@@ -238,12 +245,14 @@ __device__ __forceinline__ void stage_tile_body(const StageParams<R>& p, const E
       (reinterpret_cast<uintptr_t>(cellbuf + CellIn<2, VISC, sizeof(R) == 4>::n * ncell) + 15) &
       ~static_cast<uintptr_t>(15));
 
-  const int nthr = (t.TJ + 1) * (t.TK + 1);
+  constexpr bool F64 = sizeof(R) == 8;
+  const int nthr = F64 ? kTileThreadsF64 : (t.TJ + 1) * (t.TK + 1);
   const bool worker = threadIdx.x < nthr;
   // threads beyond the tile act as a copy of thread 0 that skips every
   // shared-memory write and every output (only the barriers need them)
   const int tid = worker ? (int)threadIdx.x : 0;
-  const int ta = tid / (t.TK + 1), tb = tid - ta * (t.TK + 1);
+  const int rowlen = F64 ? t.TK : t.TK + 1;   // FP64: thread = cell; FP32: thread = interface position
+  const int ta = tid / rowlen, tb = tid - ta * rowlen;
   const int tkt = bidx % t.ntk;
   bidx /= t.ntk;
   const int tjt = bidx % t.ntj;
@@ -281,12 +290,10 @@ __device__ __forceinline__ void stage_tile_body(const StageParams<R>& p, const E
   const int vend = worker ? NV : 0;   // vectors this thread stages: w = tid, tid + nthr, ... < vend
   // FP64 also: the cells of them that a plane needs -- an output plane the
   // tile with its halo (no corners), the two planes on either side of the
-  // chunk only the tile's own columns (their x-stencil).  The conversion to v
-  // costs a square root and a division of a cell on the narrow FP64 pipe, and
-  // with few planes to a chunk most of the box is not needed: the stage of a
-  // 33 x 33 x 9 ideal event 38.7 -> 35.6 us; FP32 converts whole vectors (the
-  // tests cost it what they save).  A thread has at most 4 vectors: (TJ + 4)
-  // box_width(TK) / 4 <= 3.5 (TJ + 1) (TK + 1).
+  // chunk only the tile's own columns (their x-stencil); vectors without any
+  // are not copied, and only these cells are converted to v, which costs a
+  // square root and a division each.  (A thread has at most one vector:
+  // (TJ + 4) box_width(TK) / 4 <= 256 for up to 256 positions.)
   unsigned need_out = 0, need_own = 0;
   for (int w = tid, sh = 0; w < vend; w += nthr, sh += 4) {
     const int bj = (4 * w) / BW, c0 = kb0 + 4 * w - bj * BW;
@@ -320,29 +327,47 @@ __device__ __forceinline__ void stage_tile_body(const StageParams<R>& p, const E
     // committed after them may still be in flight): its u~ -> (u~^tau, v) in
     // place, then one barrier makes the whole plane visible
     cp_async_wait_prior();
-    unsigned mask = out_plane ? need_out : need_own;
-    for (int w = tid; w < vend; w += nthr) {   // the cells of its vectors
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        if constexpr (sizeof(R) == 8) {
-          const bool skip = !(mask & 1u);
-          mask >>= 1;
-          if (skip) continue;
+    if constexpr (F64) {
+      __syncthreads();
+      const int wide = t.TK + 4, inner = t.TJ * wide;
+      const int nconv = out_plane ? inner + 4 * t.TK : ncell;
+      for (int i = tid; i < nconv; i += nthr) {
+        int r, c;   // box row and column
+        if (!out_plane) {
+          r = i / t.TK;
+          c = coff + i - r * t.TK;
+          r += 2;
+        } else if (i < inner) {   // the tile's rows with their eta halo
+          r = i / wide;
+          c = coff - 2 + i - r * wide;
+          r += 2;
+        } else {                  // two halo rows on either side
+          r = (i - inner) / t.TK;
+          c = coff + i - inner - r * t.TK;
+          if (r >= 2) r += t.TJ;
         }
-        const int q = 4 * w + i;
+        const int q = r * BW + c;
         const R ux = box[L::V * NB + q], uy = box[(L::V + 1) * NB + q], ue = box[(L::V + 2) * NB + q];
-        const R a = R(1) + ux * ux + uy * uy + ue * ue;
         R ut, iu;
-        if constexpr (sizeof(R) == 8) {
-          sqrt_and_inverse(a, ut, iu);
-        } else {
-          ut = sqrt(a);
-          iu = R(1) / ut;
-        }
+        sqrt_and_inverse(R(1) + ux * ux + uy * uy + ue * ue, ut, iu);
         box[L::UT * NB + q] = ut;
         box[L::V * NB + q] = ux * iu;
         box[(L::V + 1) * NB + q] = uy * iu;
         box[(L::V + 2) * NB + q] = ue * iu;
+      }
+    } else {
+      for (int w = tid; w < vend; w += nthr) {   // the cells of its vectors
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int q = 4 * w + i;
+          const R ux = box[L::V * NB + q], uy = box[(L::V + 1) * NB + q], ue = box[(L::V + 2) * NB + q];
+          const R ut = sqrt(R(1) + ux * ux + uy * uy + ue * ue);
+          const R iu = R(1) / ut;
+          box[L::UT * NB + q] = ut;
+          box[L::V * NB + q] = ux * iu;
+          box[(L::V + 1) * NB + q] = uy * iu;
+          box[(L::V + 2) * NB + q] = ue * iu;
+        }
       }
     }
     __syncthreads();
@@ -354,16 +379,33 @@ __device__ __forceinline__ void stage_tile_body(const StageParams<R>& p, const E
     cp_async_commit();
     // ---- 2. every y- and eta-interface of an output plane, once
     if (out_plane) {
-      R H[NQ];
-      if (worker && tb < t.TK) {   // y-interface between rows ta-1 and ta of column tb
-        box_interface<R, VISC>(box, NB, (ta + 2) * BW + tb + coff, BW, 2, taus, H);
+      if constexpr (F64) {
+        for (int i = tid; i < NHY + NHK; i += nthr) {
+          R H[NQ];
+          if (i < NHY) {   // y-interface between rows r-1 and r of column c
+            const int r = i / t.TK, c = i - r * t.TK;
+            box_interface<R, VISC>(box, NB, (r + 2) * BW + c + coff, BW, 2, taus, H);
 #pragma unroll
-        for (int q = 0; q < NQ; ++q) Hy[q * NHY + ta * t.TK + tb] = H[q];
-      }
-      if (worker && ta < t.TJ) {   // eta-interface between columns tb-1 and tb of row ta
-        box_interface<R, VISC>(box, NB, (ta + 2) * BW + tb + coff, 1, 3, taus, H);
+            for (int q = 0; q < NQ; ++q) Hy[q * NHY + i] = H[q];
+          } else {         // eta-interface between columns c-1 and c of row r
+            const int h = i - NHY, r = h / (t.TK + 1), c = h - r * (t.TK + 1);
+            box_interface<R, VISC>(box, NB, (r + 2) * BW + c + coff, 1, 3, taus, H);
 #pragma unroll
-        for (int q = 0; q < NQ; ++q) Hk[q * NHK + ta * (t.TK + 1) + tb] = H[q];
+            for (int q = 0; q < NQ; ++q) Hk[q * NHK + h] = H[q];
+          }
+        }
+      } else {
+        R H[NQ];
+        if (worker && tb < t.TK) {   // y-interface between rows ta-1 and ta of column tb
+          box_interface<R, VISC>(box, NB, (ta + 2) * BW + tb + coff, BW, 2, taus, H);
+#pragma unroll
+          for (int q = 0; q < NQ; ++q) Hy[q * NHY + ta * t.TK + tb] = H[q];
+        }
+        if (worker && ta < t.TJ) {   // eta-interface between columns tb-1 and tb of row ta
+          box_interface<R, VISC>(box, NB, (ta + 2) * BW + tb + coff, 1, 3, taus, H);
+#pragma unroll
+          for (int q = 0; q < NQ; ++q) Hk[q * NHK + ta * (t.TK + 1) + tb] = H[q];
+        }
       }
       __syncthreads();
     }
