@@ -791,14 +791,7 @@ __global__ void __launch_bounds__(kBlock) convert_kernel(const ConvertSet<R> x, 
     if (c >= npad) return;
     long long row;
     int k;
-    if (npad <= (1ll << 31)) {
-      const unsigned r = (unsigned)c / (unsigned)nep;
-      row = r;
-      k = (int)((unsigned)c - r * (unsigned)nep);
-    } else {
-      row = c / nep;
-      k = (int)(c - row * nep);
-    }
+    split_index(c, nep, row, k);
     d[c] = s && k < ne ? (R)s[row * ne + k] : R(0);
   }
 }

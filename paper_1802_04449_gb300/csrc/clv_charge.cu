@@ -52,10 +52,12 @@ __global__ void __launch_bounds__(kBlock) charge_stage_kernel(const StageParams<
   enter_step_kernel();
   const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= p.N) return;
-  const int k = (int)(c % p.nep);
+  long long row, plane;
+  int k, j;
+  split_index(c, p.nep, row, k);
   if (k >= p.ne) return;   // padding slot of the eta pitch
-  const long long row = c / p.nep;
-  const int j = (int)(row % p.ny), i = (int)(row / p.ny);
+  split_index(row, p.ny, plane, j);
+  const int i = (int)plane;
   const TauFactors<R> ts = tau_factors(p, STAGE);
   const R inv_dl[3] = {p.inv_dl[0], p.inv_dl[1], ts.inv_de};
   R S = R(0);

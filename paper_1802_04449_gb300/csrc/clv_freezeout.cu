@@ -53,11 +53,12 @@ __device__ __forceinline__ long long corner_offset(const FoArgs<R>& a, int i, in
   return ((long long)(i + (q >> 1 & 1)) * a.ny + (j + (q >> 2 & 1))) * a.pitch + (k + (q >> 3 & 1));
 }
 
-__device__ __forceinline__ void decode_cube(long long c, int cy, int ce, int& i, int& j, int& k) {
-  k = (int)(c % ce);
-  const long long t = c / ce;
-  j = (int)(t % cy);
-  i = (int)(t / cy);
+// (the number of hypercubes is below 2^31)
+__device__ __forceinline__ void decode_cube(unsigned c, int cy, int ce, int& i, int& j, int& k) {
+  const unsigned t = c / (unsigned)ce;
+  k = (int)(c - t * (unsigned)ce);
+  i = (int)(t / (unsigned)cy);
+  j = (int)(t - (unsigned)i * (unsigned)cy);
 }
 
 template <typename R>
@@ -67,7 +68,7 @@ __global__ void __launch_bounds__(kThreads) fo_classify_kernel(FoArgs<R> a, unsi
   int crossed = 0;
   if (c < a.ncube) {
     int i, j, k;
-    decode_cube(c, a.cy, a.ce, i, j, k);
+    decode_cube((unsigned)c, a.cy, a.ce, i, j, k);
     int nin = 0;
 #pragma unroll
     for (int q = 0; q < 16; ++q) nin += a.e[q & 1][corner_offset(a, i, j, k, q)] >= a.ef;
@@ -299,7 +300,7 @@ __global__ void __launch_bounds__(kElemThreads, sizeof(R) == 4 ? 4 : 2) fo_eleme
   for (long long e = (long long)blockIdx.x * (kElemThreads / 32) + (threadIdx.x >> 5); e < n; e += nwarps) {
     const int c = list[e];
     int i, j, k;
-    decode_cube(c, a.cy, a.ce, i, j, k);
+    decode_cube((unsigned)c, a.cy, a.ce, i, j, k);
     R fq = 0;
     if (lane < 16) fq = a.e[lane & 1][corner_offset(a, i, j, k, lane)] - a.ef;
     R f[5];

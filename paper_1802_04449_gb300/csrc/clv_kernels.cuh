@@ -169,6 +169,19 @@ __device__ __forceinline__ int wrap_index(int i, int n, int periodic) {
   return i < 0 ? 0 : (i >= n ? n - 1 : i);
 }
 
+// Row c / n and place c % n in it of index c, by a 32-bit division where c
+// allows it (a 64-bit one is ~70 instructions).
+__device__ __forceinline__ void split_index(long long c, int n, long long& row, int& rest) {
+  if (c < (1ll << 31)) {
+    const unsigned r = (unsigned)c / (unsigned)n;
+    row = r;
+    rest = (int)((unsigned)c - r * (unsigned)n);
+  } else {
+    row = c / n;
+    rest = (int)(c - row * n);
+  }
+}
+
 template <typename R> __device__ __forceinline__ R ldg(const R* p) { return __ldg(p); }
 
 template <typename R> struct SolveTraits;
@@ -455,15 +468,18 @@ template <typename R, int STAGE, bool VISC, bool STATS>
 __global__ void __launch_bounds__(kBlock) stage_kernel(const StageParams<R> p) {
   enter_step_kernel();
   const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const bool active = c < p.N && (int)(c % p.nep) < p.ne;   // padding slots of the eta rows do no work
+  long long row;
+  int k;
+  split_index(c, p.nep, row, k);
+  const bool active = c < p.N && k < p.ne;   // padding slots of the eta rows do no work
   double my_T0 = 0.0;
   double my_e = 0.0;
   bool f_rescaled = false, f_fail = false, f_polished = false, f_nonfinite = false, f_nonconv = false;
   if (active) {
-    const int k = (int)(c % p.nep);
-    const long long t = c / p.nep;
-    const int j = (int)(t % p.ny);
-    const int i = (int)(t / p.ny);
+    long long ii0;
+    int j;
+    split_index(row, p.ny, ii0, j);
+    const int i = (int)ii0;
     constexpr int NR = NRec<VISC>::n;
     constexpr int NQ = VISC ? 14 : 4;
     constexpr int IU = VISC ? 14 : 4, IV = IU + 1;
@@ -1056,6 +1072,17 @@ static __global__ void __launch_bounds__(kBlock) scan_counts_kernel(const unsign
   for (int i = lo; i < hi; ++i) { offsets[i] = run; run += counts[i]; }
 }
 
+// A normal float or a zero as a double by its bits: the FP64 pipe, which does
+// conversions, has 2 lanes an SM and cycle and would bound an export.
+__device__ __forceinline__ double widen(float x) {
+  const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
+  if (m - 0x00800000u < 0x7f000000u)
+    return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(b << 29));
+  if (m == 0) return __hiloint2double((int)b, 0);
+  return (double)x;
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+
 // T~^{tau mu} = tau [(e + P) u^tau u^mu - P g~^{tau mu} + pi~^{tau mu}], in
 // FP64 from the stored primitives; written as R, and (FP32 path, lo != null)
 // as float-float pairs: high parts T, low parts lo
@@ -1064,18 +1091,19 @@ __global__ void __launch_bounds__(kBlock) tilde_T_kernel(Prim<R> pr, Ptr10<R> pi
                                                          Ptr10<R> lo, bool with_lo, double taus, long long N) {
   const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= N) return;
-  const double e = pr.e[c], P = pr.P[c];
-  const double u1 = pr.u[0][c], u2 = pr.u[1][c], u3 = pr.u[2][c];
+  // FP32: conversions off the FP64 pipe, which bounds the kernel
+  const double e = widen(pr.e[c]), P = widen(pr.P[c]);
+  const double u1 = widen(pr.u[0][c]), u2 = widen(pr.u[1][c]), u3 = widen(pr.u[2][c]);
   const double u0 = sqrt(1.0 + u1 * u1 + u2 * u2 + u3 * u3);
   const double w = (e + P) * u0;
   double a0 = w * u0 - P, a1 = w * u1, a2 = w * u2, a3 = w * u3;
-  if (with_pi) { a0 += (double)pi.p[0][c]; a1 += (double)pi.p[1][c]; a2 += (double)pi.p[2][c]; a3 += (double)pi.p[3][c]; }
+  if (with_pi) { a0 += widen(pi.p[0][c]); a1 += widen(pi.p[1][c]); a2 += widen(pi.p[2][c]); a3 += widen(pi.p[3][c]); }
   const double v[4] = {taus * a0, taus * a1, taus * a2, taus * a3};
 #pragma unroll
   for (int m = 0; m < 4; ++m) {
     const R hi = (R)v[m];
     T.p[m][c] = hi;
-    if (with_lo) lo.p[m][c] = (R)(v[m] - (double)hi);
+    if (with_lo) lo.p[m][c] = (R)(v[m] - widen(hi));
   }
 }
 
@@ -1116,11 +1144,10 @@ __global__ void __launch_bounds__(kBlock) extrapolate_prev_kernel(Prim<R> cur, P
 // Cell c of the compact order (nx, ny, neta) <-> its slot in the padded
 // layout, whose eta rows have a pitch nep >= neta (a multiple of 4).
 __device__ __forceinline__ long long padded_index(long long c, int ne, int nep) {
-  if (c < (1ll << 31)) {   // 32-bit division
-    const unsigned row = (unsigned)c / (unsigned)ne;
-    return (long long)row * nep + ((unsigned)c - row * (unsigned)ne);
-  }
-  return (c / ne) * nep + c % ne;
+  long long row;
+  int k;
+  split_index(c, ne, row, k);
+  return row * nep + k;
 }
 
 // fields as compact doubles, field blockIdx.y to dst + blockIdx.y N; a
@@ -1130,17 +1157,6 @@ template <typename R> struct ExportSet {
   const R *hi[kMaxExport], *lo[kMaxExport];
   double* dst[kMaxExport];
 };
-// A normal float or a zero as a double by its bits: the FP64 pipe, which does
-// conversions, has 2 lanes an SM and cycle and would bound an export.
-__device__ __forceinline__ double widen(float x) {
-  const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
-  if (m - 0x00800000u < 0x7f000000u)
-    return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(b << 29));
-  if (m == 0) return __hiloint2double((int)b, 0);
-  return (double)x;
-}
-__device__ __forceinline__ double widen(double x) { return x; }
-
 // Cells of a thread in the initial-state and export transfers: loads in flight
 // for the bandwidth.  Export of 18 fields of 261 x 261 x 121 cells: 0.80 ms
 // with one converted by the FP64 pipe.
