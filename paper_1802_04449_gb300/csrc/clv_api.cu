@@ -230,16 +230,11 @@ int tile_occupancy(const clv_config* c, int threads, size_t smem) {
 // dependent instructions whatever the tile, plus the box's cells (97 x 97 x 41
 // viscous stage 1: 7 x 22 tiles 4.8 us, 12 x 21 5.3, 16 x 21 6.0, two of 7 x 21
 // 5.8); the 4 halo planes, without y and eta interfaces, cost about 3.
-// FP64: warp passes of the busiest quarter of the SM (TileBound) times the FP64
-// instructions of an interface, of a cell with its x-interface and of a
-// conversion.
+// FP64: the cells over a chain that is the longer part of an ideal tile (97 x
+// 97 x 41 viscous: 7 x 14 tiles 41 us, 9 x 14 45, 10 x 14 53; 33 x 33 x 9 ideal,
+// stages of one plane: 9 x 9 27 us, 13 x 9 30).
 double plane_cost(const clv_config* c, int TJ, int TK, int occ) {
-  if (c->precision == CLV_FP64) {
-    auto passes = [](int n) { return ((n + 31) / 32 + 3) / 4; };
-    const bool visc = c->eta_over_s > 0.0;
-    return (visc ? 110.0 : 65.0) * passes((TJ + 1) * TK + TJ * (TK + 1)) + (visc ? 240.0 : 130.0) * passes(TJ * TK) +
-           17.0 * passes(TJ * (TK + 4) + 4 * TK) + 30.0;
-  }
+  if (c->precision == CLV_FP64) return (c->eta_over_s > 0.0 ? 91.0 : 221.0) + occ * (double)(TJ * TK);
   return 620.0 + occ * (double)((TJ + 4) * box_width(TK));
 }
 inline double halo_planes(const clv_config* c) { return c->precision == CLV_FP64 ? 1.2 : 3.0; }

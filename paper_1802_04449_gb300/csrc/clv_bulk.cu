@@ -65,6 +65,7 @@ template <typename R, int STAGE>
 __global__ void __launch_bounds__(kBlock) bulk_stage_kernel(const StageParams<R> p, const R* __restrict__ Pin,
                                                             const R* Pn, R* Pout,   // Pn == Pout in stage 2
                                                             const R inv_5zs_hbarc) {
+  release_next_kernel();
   enter_step_kernel();
   const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= p.N) return;

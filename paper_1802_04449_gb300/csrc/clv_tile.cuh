@@ -208,13 +208,11 @@ __device__ __forceinline__ void box_interface(const R* box, int NB, int c, int s
 // threads.  FP32: a thread per position, 384 (12 warps) fit the register file
 // at the 168 registers that bound allows; a CTA of at most 192 threads then
 // leaves room for a second one on the SM, when its shared memory fits too.
-// FP64: always 256 threads (8 warps of 255 registers).  A quarter of the SM
-// issues an FP64 warp instruction over 64 cycles whatever its active lanes, so
-// what a plane costs is the warp passes of the busiest quarter: the conversions
-// and the interfaces are spread over all warps as tasks and the cells over the
-// first threads, instead of a thread per position doing one of each (a 10 x 14
-// tile: six warps, two on two of the quarters, three of them converting four
-// cells in turn).
+// FP64: always 256 threads (8 warps of 255 registers): the conversions and the
+// interfaces are spread over all of them as tasks and the cells over the first
+// ones, instead of a thread per position doing one of each (a thread converted
+// up to four cells of each plane in turn, on a pipe of 2 lanes an SM and cycle:
+// the stage of a 33 x 33 x 9 ideal event 35.0 -> 26.9 us).
 #ifndef CLV_TILE_MAX_THREADS
 #define CLV_TILE_MAX_THREADS 384
 #endif
