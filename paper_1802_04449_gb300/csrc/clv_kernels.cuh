@@ -754,15 +754,17 @@ __global__ void __launch_bounds__(kBlock) stage_kernel(const StageParams<R> p) {
 // the new T~^{tau mu} and pi~^{tau mu}, solves for (eps, u~) warm-started
 // from the stage velocity, writes P and c_s, zeroes pi~ in vacuum cells, and
 // (STATS) reduces sum T~^{tau tau} and max eps.
-// at least four 256-thread blocks per SM in FP32 (at most 64 registers): the
-// dependent table lookups of the root solve need the occupancy
-template <typename R>
+// blocks of 256 threads (or as many smaller ones) per SM: the dependent table
+// lookups of the root solve need the occupancy.  In FP32 six, with 42 registers
+// and a small spill, are 10% faster than four (261 x 261 x 121 cells: 239 -> 213
+// us a launch); with the network, which then spills more, four are best
+template <typename R, int GUESS>
 struct RecoverMinBlocks {
-  static constexpr int value = sizeof(R) == 4 ? 4 : 3;
+  static constexpr int value = sizeof(R) == 8 ? 3 : GUESS == kGuessMlp || GUESS == kGuessMlpAll ? 4 : 6;
 };
 
 template <typename R, bool VISC, bool STATS, int GUESS = kGuessPrevious>
-__global__ void __launch_bounds__(kBlock, RecoverMinBlocks<R>::value) recover_kernel(const StageParams<R> p) {
+__global__ void __launch_bounds__(kBlock, RecoverMinBlocks<R, GUESS>::value) recover_kernel(const StageParams<R> p) {
   release_next_kernel();
   enter_step_kernel();
   const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
