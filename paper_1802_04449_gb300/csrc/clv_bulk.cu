@@ -39,24 +39,23 @@ template <typename R>
 __device__ __forceinline__ BulkCell<R> bulk_cell(const StageParams<R>& p, const R* __restrict__ Pin, long long s,
                                                  int axis) {
   const R ux = p.pr.u[0][s], uy = p.pr.u[1][s], ue = p.pr.u[2][s];
-  const R ut = sqrt(R(1) + ux * ux + uy * uy + ue * ue);
+  R ut, iu;
+  sqrt_and_inverse(R(1) + ux * ux + uy * uy + ue * ue, ut, iu);
   const R ua = axis == 0 ? ux : (axis == 1 ? uy : ue);
-  return BulkCell<R>{ut, ua / ut, Pin[s], p.pr.cs[s], ua};
+  return BulkCell<R>{ut, ua * iu, Pin[s], p.pr.cs[s], ua};
 }
 
 // flux v^a u~^tau Pi at the interface between cells b and c from cells a, b, c, d
 template <typename R>
 __device__ __forceinline__ R bulk_flux(const BulkCell<R>& a, const BulkCell<R>& b, const BulkCell<R>& c,
                                        const BulkCell<R>& d) {
-  const R utL = b.ut + R(0.5) * minmod(b.ut - a.ut, c.ut - b.ut);
+  const R utL = b.ut + R(0.5) * minmod(c.ut - b.ut, b.ut - a.ut);
   const R utR = c.ut - R(0.5) * minmod(c.ut - b.ut, d.ut - c.ut);
-  const R vL = b.v + R(0.5) * minmod(b.v - a.v, c.v - b.v);
+  const R vL = b.v + R(0.5) * minmod(c.v - b.v, b.v - a.v);
   const R vR = c.v - R(0.5) * minmod(c.v - b.v, d.v - c.v);
-  const R PL = b.Pi + R(0.5) * minmod(b.Pi - a.Pi, c.Pi - b.Pi);
+  const R PL = b.Pi + R(0.5) * minmod(c.Pi - b.Pi, b.Pi - a.Pi);
   const R PR = c.Pi - R(0.5) * minmod(c.Pi - b.Pi, d.Pi - c.Pi);
-  const R lL = (fabs(vL) + b.cs) / (R(1) + fabs(vL) * b.cs);
-  const R lR = (fabs(vR) + c.cs) / (R(1) + fabs(vR) * c.cs);
-  const R lam = lL > lR ? lL : lR;
+  const R lam = signal_speed(vL, b.cs, vR, c.cs);
   const R QL = utL * PL, QR = utR * PR;
   return R(0.5) * (vL * QL + vR * QR) - R(0.5) * lam * (QR - QL);
 }

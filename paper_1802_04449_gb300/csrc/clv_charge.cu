@@ -27,22 +27,21 @@ template <typename R>
 __device__ __forceinline__ ChargeCell<R> charge_cell(const StageParams<R>& p, const R* __restrict__ Nin, long long s,
                                                      int axis) {
   const R ux = p.pr.u[0][s], uy = p.pr.u[1][s], ue = p.pr.u[2][s];
-  const R ut = sqrt(R(1) + ux * ux + uy * uy + ue * ue);
+  R ut, iu;
+  sqrt_and_inverse(R(1) + ux * ux + uy * uy + ue * ue, ut, iu);
   const R ua = axis == 0 ? ux : (axis == 1 ? uy : ue);
-  return ChargeCell<R>{Nin[s], ua / ut, p.pr.cs[s]};
+  return ChargeCell<R>{Nin[s], ua * iu, p.pr.cs[s]};
 }
 
 // flux at the interface between cells b and c from cells a, b, c, d
 template <typename R>
 __device__ __forceinline__ R charge_flux(const ChargeCell<R>& a, const ChargeCell<R>& b, const ChargeCell<R>& c,
                                          const ChargeCell<R>& d) {
-  const R NL = b.N + R(0.5) * minmod(b.N - a.N, c.N - b.N);
+  const R NL = b.N + R(0.5) * minmod(c.N - b.N, b.N - a.N);
   const R NR = c.N - R(0.5) * minmod(c.N - b.N, d.N - c.N);
-  const R vL = b.v + R(0.5) * minmod(b.v - a.v, c.v - b.v);
+  const R vL = b.v + R(0.5) * minmod(c.v - b.v, b.v - a.v);
   const R vR = c.v - R(0.5) * minmod(c.v - b.v, d.v - c.v);
-  const R lL = (fabs(vL) + b.cs) / (R(1) + fabs(vL) * b.cs);
-  const R lR = (fabs(vR) + c.cs) / (R(1) + fabs(vR) * c.cs);
-  const R lam = lL > lR ? lL : lR;
+  const R lam = signal_speed(vL, b.cs, vR, c.cs);
   return R(0.5) * (vL * NL + vR * NR) - R(0.5) * lam * (NR - NL);
 }
 

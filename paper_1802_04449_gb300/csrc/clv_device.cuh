@@ -428,6 +428,21 @@ __device__ __forceinline__ void sqrt_and_inverse(double a, double& root, double&
   root = fma(fma(-r, r, a), 0.5 * inv, r);
 }
 
+__device__ __forceinline__ void sqrt_and_inverse(float a, float& root, float& inv) {
+  inv = rsqrtf(a);
+  const float r = mul_rn(a, inv);
+  root = fmaf(fmaf(-r, r, a), 0.5f * inv, r);
+}
+
+// max of (|v| + c_s)/(1 + |v| c_s) of two sides, the larger found by
+// cross-multiplication: one division
+template <typename R> __device__ __forceinline__ R signal_speed(R vl, R csl, R vr, R csr) {
+  const R al = fabs(vl), ar = fabs(vr);
+  const R nl = al + csl, dl = R(1) + al * csl, nr = ar + csr, dr = R(1) + ar * csr;
+  const bool rs = nr * dl > nl * dr;
+  return (rs ? nr : nl) / (rs ? dr : dl);
+}
+
 // minmod(a, b): 0 unless a and b share a sign, else the one of smaller
 // magnitude (the value is a, b or 0 exactly).  FP32: b clamped to the
 // interval between 0 and a, four min/max operations on the ALU pipe.  FP64:

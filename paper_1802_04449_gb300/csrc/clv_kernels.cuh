@@ -219,12 +219,7 @@ __device__ __forceinline__ void interface_flux(const R* L, const R* Rr, R csl, R
   constexpr int NQ = VISC ? 14 : 4;
   constexpr int IU = VISC ? 14 : 4, IV = IU + 1, IP = IU + 2;
   const R vl = L[IV], vr = Rr[IV];
-  const R al = fabs(vl), ar = fabs(vr);
-  // lam = max of (|v| + c_s)/(1 + |v| c_s) of the two sides, the larger one
-  // found by cross-multiplication: one division
-  const R nl = al + csl, dl = R(1) + al * csl, nr = ar + csr, dr = R(1) + ar * csr;
-  const bool rs = nr * dl > nl * dr;
-  const R lam = (rs ? nr : nl) / (rs ? dr : dl);
+  const R lam = signal_speed(vl, csl, vr, csr);
   // H = (F_l + F_r)/2 - lam (Q_r - Q_l)/2 with F = v Q + tau X regrouped as
   // wl Q_l + wr Q_r + tau (X_l + X_r)/2, wl = (v_l + lam)/2, wr = (v_r - lam)/2
   const R wl = R(0.5) * (vl + lam), wr = R(0.5) * (vr - lam);
