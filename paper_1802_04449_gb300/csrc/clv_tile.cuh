@@ -249,7 +249,15 @@ __device__ __forceinline__ void stage_tile_body(const StageParams<R>& p, const E
   // threads beyond the tile act as a copy of thread 0 that skips every
   // shared-memory write and every output (only the barriers need them)
   const int tid = worker ? (int)threadIdx.x : 0;
-  const int rowlen = F64 ? t.TK : t.TK + 1;   // FP64: thread = cell; FP32: thread = interface position
+  // Thread = cell (ta, tb) below ncell, = y-interface (ta, tb) below NHY and
+  // (FP32) = eta-interface tid, in rows of TK + 1, below NHK: each list fills
+  // whole warps, and the last threads, with least to do, take the staging
+  // first (8 x 41 tiles, 97 x 97 x 41: stage 1 67.8 -> 65.7 us against a thread
+  // per position).  A batch in FP32 keeps a thread per position of (TJ+1) rows of
+  // TK + 1: in the loop over its items the other one spills 200 bytes (twelve
+  // events, 40 steps: 65 -> 79 ms).
+  constexpr bool POSITIONS = !F64 && BATCH;
+  const int rowlen = POSITIONS ? t.TK + 1 : t.TK;
   const int ta = tid / rowlen, tb = tid - ta * rowlen;
   const int tkt = bidx % t.ntk;
   bidx /= t.ntk;
@@ -259,11 +267,16 @@ __device__ __forceinline__ void stage_tile_body(const StageParams<R>& p, const E
   const int kb0 = ((k0 - 2) >> 2) << 2;   // first box column: k0 - 2 rounded down to a multiple of 4
   const int coff = k0 - kb0;              // box column of the tile's first column (2..5)
   const int x1 = min(x0 + t.CX, ev.nx);
-  const bool is_cell = worker && ta < t.TJ && tb < t.TK;
+  const bool is_cell = worker && (POSITIONS ? ta < t.TJ && tb < t.TK : tid < ncell);
   const int j = j0 + ta, k = k0 + tb;
   const bool active = is_cell && j < ev.ny && k < ev.ne;
-  const int cid = ta * t.TK + tb;                  // cell slot (valid when is_cell)
+  const int cid = ta * t.TK + tb;                  // slot of cell and of y-interface (ta, tb)
   const int center = (ta + 2) * BW + (tb + coff);  // box cell of (ta, tb)
+  int ecell = 0;   // !POSITIONS: box cell right of eta-interface tid
+  if constexpr (!POSITIONS) {
+    const int r = tid / (t.TK + 1);
+    ecell = (r + 2) * BW + (tid - r * (t.TK + 1) + coff);
+  }
   const TauFactors<R> ts = tau_factors(p, STAGE);
   const R taus = ts.taus;
   const R inv_dx = ev.inv_dx;
@@ -285,7 +298,8 @@ __device__ __forceinline__ void stage_tile_body(const StageParams<R>& p, const E
 
 
   // in-plane offsets of this thread's box vectors (only this thread uses them)
-  const int vend = worker ? NV : 0;   // vectors this thread stages: w = tid, tid + nthr, ... < vend
+  const int vend = worker ? NV : 0;   // vectors this thread stages: w = w0, w0 + nthr, ... < vend
+  const int w0 = POSITIONS ? tid : nthr - 1 - tid;
   // FP64 also: the cells of them that a plane needs -- an output plane the
   // tile with its halo (no corners), the two planes on either side of the
   // chunk only the tile's own columns (their x-stencil); vectors without any
@@ -293,7 +307,7 @@ __device__ __forceinline__ void stage_tile_body(const StageParams<R>& p, const E
   // square root and a division each.  (A thread has at most one vector:
   // (TJ + 4) box_width(TK) / 4 <= 256 for up to 256 positions.)
   unsigned need_out = 0, need_own = 0;
-  for (int w = tid, sh = 0; w < vend; w += nthr, sh += 4) {
+  for (int w = w0, sh = 0; w < vend; w += nthr, sh += 4) {
     const int bj = (4 * w) / BW, c0 = kb0 + 4 * w - bj * BW;
     for (int i = 0; i < 4 && sizeof(R) == 8; ++i) {
       const int col = c0 + i - k0;
@@ -315,7 +329,7 @@ __device__ __forceinline__ void stage_tile_body(const StageParams<R>& p, const E
   // (the per-cell inputs of its next output cell), each possibly empty, so
   // that waiting for all but the newest group lands exactly the one needed.
   stage_plane_async<R, VISC>(p, boxbuf + ((x0 - 2) & 1) * NF * NB, vend, ev.off + xplane(x0 - 2) * plane, voff,
-                             need_own, tid, nthr, NB);
+                             need_own, w0, nthr, NB);
   cp_async_commit();
   cp_async_commit();   // no cell group before the first plane
   for (int pl = x0 - 2; pl <= x1 + 1; ++pl) {
@@ -354,7 +368,7 @@ __device__ __forceinline__ void stage_tile_body(const StageParams<R>& p, const E
         box[(L::V + 2) * NB + q] = ue * iu;
       }
     } else {
-      for (int w = tid; w < vend; w += nthr) {   // the cells of its vectors
+      for (int w = w0; w < vend; w += nthr) {   // the cells of its vectors
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           const int q = 4 * w + i;
@@ -373,7 +387,7 @@ __device__ __forceinline__ void stage_tile_body(const StageParams<R>& p, const E
     if (pl + 1 <= x1 + 1)
       stage_plane_async<R, VISC>(p, boxbuf + ((pl + 1) & 1) * NF * NB, vend,
                                  ev.off + xplane(pl + 1) * plane, voff,
-                                 pl + 1 >= x0 && pl + 1 < x1 ? need_out : need_own, tid, nthr, NB);
+                                 pl + 1 >= x0 && pl + 1 < x1 ? need_out : need_own, w0, nthr, NB);
     cp_async_commit();
     // ---- 2. every y- and eta-interface of an output plane, once
     if (out_plane) {
@@ -394,15 +408,21 @@ __device__ __forceinline__ void stage_tile_body(const StageParams<R>& p, const E
         }
       } else {
         R H[NQ];
-        if (worker && tb < t.TK) {   // y-interface between rows ta-1 and ta of column tb
-          box_interface<R, VISC>(box, NB, (ta + 2) * BW + tb + coff, BW, 2, taus, H);
+        if (worker && (POSITIONS ? tb < t.TK : tid < NHY)) {   // y-interface between rows ta-1 and ta of column tb
+          box_interface<R, VISC>(box, NB, center, BW, 2, taus, H);
 #pragma unroll
           for (int q = 0; q < NQ; ++q) Hy[q * NHY + ta * t.TK + tb] = H[q];
         }
-        if (worker && ta < t.TJ) {   // eta-interface between columns tb-1 and tb of row ta
-          box_interface<R, VISC>(box, NB, (ta + 2) * BW + tb + coff, 1, 3, taus, H);
+        if constexpr (POSITIONS) {
+          if (worker && ta < t.TJ) {   // eta-interface between columns tb-1 and tb of row ta
+            box_interface<R, VISC>(box, NB, center, 1, 3, taus, H);
 #pragma unroll
-          for (int q = 0; q < NQ; ++q) Hk[q * NHK + ta * (t.TK + 1) + tb] = H[q];
+            for (int q = 0; q < NQ; ++q) Hk[q * NHK + ta * (t.TK + 1) + tb] = H[q];
+          }
+        } else if (worker && tid < NHK) {   // eta-interface tid
+          box_interface<R, VISC>(box, NB, ecell, 1, 3, taus, H);
+#pragma unroll
+          for (int q = 0; q < NQ; ++q) Hk[q * NHK + tid] = H[q];
         }
       }
       __syncthreads();
