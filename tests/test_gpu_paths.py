@@ -17,7 +17,7 @@ FIELDS = ["eps", "ux", "uy", "ueta", "Ttt", "pixx", "piee"]
 
 @pytest.mark.parametrize("prec,shapes", [
     (clv.CLV_FP64, [(1, 1), (1, 45), (2, 13), (8, 16), (10, 14), (30, 3), (37, 2)]),
-    (clv.CLV_FP32, [(1, 1), (1, 45), (8, 41), (7, 45), (31, 11), (37, 9)])])
+    (clv.CLV_FP32, [(1, 1), (1, 45), (8, 41), (6, 45), (28, 11), (37, 7)])])
 @pytest.mark.parametrize("eta_over_s", [0.0, 0.08])
 def test_tiles_at_the_limits_of_their_tasks(prec, shapes, eta_over_s):
     case = I.hotspot_event(nx=9, ny=37, neta=45, n_spots=60, seed=5, eta_over_s=eta_over_s)
