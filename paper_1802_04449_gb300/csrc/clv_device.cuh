@@ -256,7 +256,16 @@ __device__ __forceinline__ RootResult solve_primitive(const EosView<R>& q, C eps
   C P, cs2, dPde;   // dPde: d(P + Pshift)/d eps, 0 on the floor (cs2 keeps the table's value)
   C v;
   bool fixed = FIXED;
-  if (vguess && *vguess > lo && *vguess < hi) {
+  // conformal EOS: f is a quadratic in v (off the pressure floor), and its root
+  // is the start, which the first Newton step then confirms
+  C vconf = C(-1);
+  if (!FIXED && q.kind == 0) {
+    const C A = C(4.0 / 3.0) * E + Pshift, disc = A * A - C(4.0 / 3.0) * (M * M);
+    if (A > C(0) && disc > C(0)) vconf = Ops::div(C(2) * M, A + Ops::sqrt_(disc));
+  }
+  if (vconf > lo && vconf < hi) {
+    v = vconf;
+  } else if (vguess && *vguess > lo && *vguess < hi) {
     v = *vguess;
   } else {
     if (FIXED) { fixed = false; maxit = 100; }  // no usable start: solve in full
