@@ -347,7 +347,7 @@ size_t layout(const clv_config* c, clv_handle* h) {
   // FP32 path: T~ as float-float pairs (StageParams), the low parts in 2 x 4 more arrays
   const bool ffT = c->precision != CLV_FP64;
   // block partials of the stats reduction: enough for the smallest recovery blocks
-  const int nblocks = (int)((N + kRecoverSmall - 1) / kRecoverSmall);
+  const int nblocks = (int)((N + kRecoverSmall - 1) / kRecoverSmall) + 1;
   size_t off = 0;
   auto take = [&](size_t bytes) { size_t o = off; off += align_up(bytes, 256); return o; };
   size_t oT0[4], oPI0[10], oT1[4], oPI1[10], oPR[kNumPrimSets][kPrimFields], oE[3];
@@ -541,9 +541,9 @@ inline int recover_block(const clv_handle* h) {
   const bool net = h->rsize == 4 && (h->guess == kGuessMlp || h->guess == kGuessMlpAll);
   return net && (h->N + kBlock - 1) / kBlock >= 2ll * h->sms ? kBlock : kRecoverSmall;
 }
-inline unsigned recover_grid(const clv_handle* h) {
+inline unsigned recover_grid(const clv_handle* h) {   // and a block for the next step's tau factors
   const int b = recover_block(h);
-  return (unsigned)((h->N + b - 1) / b);
+  return (unsigned)((h->N + b - 1) / b + 1);
 }
 
 template <typename R, bool VISC, bool STATS> void launch_recover(clv_handle* h, const StageParams<R>& p) {

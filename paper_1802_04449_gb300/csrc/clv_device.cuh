@@ -26,13 +26,49 @@ __host__ __device__ constexpr int sym_index(int m, int n) {
 }
 __host__ __device__ constexpr double metric_sign(int m) { return m == 0 ? 1.0 : -1.0; }
 
+// ln x of a positive normal double in 12 FP64 operations (the pipe has 2 lanes an
+// SM and cycle), table-driven as in P. T. P. Tang, ACM TOMS 16 (1990) 378: x = 2^ex m, m in [1, 2)
+// in one of 64 intervals with r = m c - 1, |r| <= 2^-7, for a c near the inverse
+// of its middle, ln x = ex ln 2 - ln c + r - r^2/2 + ... + r^7/7 (the rest is
+// below 2e-18).  Subnormals give about -709, zero and negatives are not passed.
+struct LogTable {
+  double c[64], mlog[64];   // c and -ln c
+};
+constexpr LogTable make_log_table() {
+  LogTable t{};
+  for (int j = 0; j < 64; ++j) {
+    const double c = (double)(float)(1.0 / (1.0 + (j + 0.5) / 64.0));
+    // -ln c = 2 artanh z, z = (1 - c)/(1 + c) < 1/3
+    const double z = (1.0 - c) / (1.0 + c), z2 = z * z;
+    double p = 0.0;
+    for (int k = 41; k >= 3; k -= 2) p = z2 * (1.0 / k + p);
+    t.c[j] = c;
+    t.mlog[j] = 2.0 * (z + z * p);
+  }
+  return t;
+}
+static __device__ const LogTable kLogTable = make_log_table();
+__device__ __forceinline__ double table_log(double x) {
+  const int hi = __double2hiint(x);
+  const int ex = (hi >> 20) - 1023, j = hi >> 14 & 63;
+  const double m = __hiloint2double((hi & 0x000fffff) | 0x3ff00000, __double2loint(x));
+  const double r = fma(m, __ldg(kLogTable.c + j), -1.0);
+  double p = fma(r, 1.0 / 7.0, -1.0 / 6.0);
+  p = fma(p, r, 1.0 / 5.0);
+  p = fma(p, r, -1.0 / 4.0);
+  p = fma(p, r, 1.0 / 3.0);
+  p = fma(p, r, -0.5);
+  p = fma(p, r * r, r);
+  return fma((double)ex, 0.69314718055994530942, __ldg(kLogTable.mlog + j)) + p;
+}
+
 template <typename R> struct Fast;
 template <> struct Fast<float> {
   static __device__ __forceinline__ float log(float x) { return __logf(x); }
   static __device__ __forceinline__ float rcp(float x) { return __frcp_rn(x); }
 };
 template <> struct Fast<double> {
-  static __device__ __forceinline__ double log(double x) { return ::log(x); }
+  static __device__ __forceinline__ double log(double x) { return table_log(x); }
   static __device__ __forceinline__ double rcp(double x) { return 1.0 / x; }
 };
 
@@ -171,6 +207,14 @@ struct RootResult {
   int rescaled;   // |M| > (1 - kMaxMoverE) E was rescaled
 };
 
+// sqrt(a) and 1/sqrt(a), a > 0, from one reciprocal square root and a
+// correction of the root (its residual a - r^2 is exact by FMA)
+__device__ __forceinline__ void sqrt_and_inverse(double a, double& root, double& inv) {
+  inv = rsqrt(a);
+  const double r = __dmul_rn(a, inv);
+  root = fma(fma(-r, r, a), 0.5 * inv, r);
+}
+
 // Division and square root for the FP64 refinement of the FP32 path: an FP32
 // seed refined by Newton steps in FP64 (fused multiply-adds only; relative
 // error ~1e-15), instead of the long FP64 division / square-root sequences.
@@ -197,6 +241,11 @@ template <typename C, typename CE> struct SolveOps {
   static __device__ __forceinline__ C div(C a, C b) { return a / b; }
   static __device__ __forceinline__ C sqrt_(C x) { return sqrt(x); }
   static __device__ __forceinline__ C rsqrt_(C x) { return C(1) / sqrt(x); }
+};
+template <> struct SolveOps<double, double> {
+  static __device__ __forceinline__ double div(double a, double b) { return a / b; }
+  static __device__ __forceinline__ double sqrt_(double x) { return sqrt(x); }
+  static __device__ __forceinline__ double rsqrt_(double x) { return rsqrt(x); }
 };
 template <> struct SolveOps<float, float> {
   static __device__ __forceinline__ float div(float a, float b) { return a / b; }
@@ -240,12 +289,19 @@ __device__ __forceinline__ RootResult solve_primitive(const EosView<R>& q, C eps
   ux = uy = ue = C(0);
   if (!(E >= eps_cut)) return rr;
   C M2 = Mx * Mx + My * My + Me * Me;
-  C M = Ops::sqrt_(M2);
+  C M, iM = C(0);   // iM: 1/M (FP64 lookups)
+  if constexpr (sizeof(CE) == 8) {
+    M = C(0);
+    if (M2 > C(0)) sqrt_and_inverse(M2, M, iM);
+  } else {
+    M = Ops::sqrt_(M2);
+  }
   C Mcap = C(1.0 - kMaxMoverE) * E;
   if (M > Mcap) {
     C s = Ops::div(Mcap, M);
     Mx *= s; My *= s; Me *= s;
     M = Mcap;
+    if constexpr (sizeof(CE) == 8) iM = Ops::div(C(1), M);
     rr.rescaled = 1;
   }
   if (M == C(0)) {
@@ -346,7 +402,9 @@ __device__ __forceinline__ RootResult solve_primitive(const EosView<R>& q, C eps
     }
   }
   C gam = Ops::rsqrt_(C(1) - v * v);
-  C s = Ops::div(gam * v, M);
+  C s;
+  if constexpr (sizeof(CE) == 8) s = gam * v * iM;
+  else s = Ops::div(gam * v, M);
   ux = s * Mx;
   uy = s * My;
   ue = s * Me;
@@ -428,14 +486,6 @@ __device__ __forceinline__ void cp_async_wait_prior() { asm volatile("cp.async.w
 // differences of equal products cancel exactly.
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
-
-// sqrt(a) and 1/sqrt(a), a >= 1, from one reciprocal square root and a
-// correction of the root (its residual a - r^2 is exact by FMA)
-__device__ __forceinline__ void sqrt_and_inverse(double a, double& root, double& inv) {
-  inv = rsqrt(a);
-  const double r = mul_rn(a, inv);
-  root = fma(fma(-r, r, a), 0.5 * inv, r);
-}
 
 __device__ __forceinline__ void sqrt_and_inverse(float a, float& root, float& inv) {
   inv = rsqrtf(a);

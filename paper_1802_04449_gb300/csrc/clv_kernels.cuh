@@ -56,7 +56,7 @@ struct TauSlot {
   double inv_taus[2];           // 1/tau_s of stages 1 and 2 (Cartesian: 1)
   TauFactors<double> d[2];
   TauFactors<float> f[2];
-  double taus_new;              // tau scale at the end of the step
+  double inv_taus_new;          // 1 over the tau scale at the end of the step
   double inv_end;               // 1/(tau + dtau)
 };
 // it: 1/tau
@@ -68,7 +68,7 @@ __device__ __forceinline__ void store_tau(TauSlot* s, double tau, double it, dou
   s->tau = tau;
   s->itau[0] = hi;
   s->itau[1] = (float)(x - (double)hi);
-  s->taus_new = cartesian ? 1.0 : end;
+  s->inv_taus_new = x;
   s->inv_end = ie;
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
@@ -297,7 +297,7 @@ template <typename R, bool VISC> struct IdealPart {
 };
 template <typename R, bool VISC>
 __device__ __forceinline__ IdealPart<R, VISC> ideal_part(const StageParams<R>& p, const R Tv[4], const R Tlv[4],
-                                                        const R pi4[4], R tn) {
+                                                        const R pi4[4]) {
   IdealPart<R, VISC> a;
   if constexpr (sizeof(R) == 4) {
     const ff itn{p.tau_dev->itau[0], p.tau_dev->itau[1]};
@@ -312,7 +312,7 @@ __device__ __forceinline__ IdealPart<R, VISC> ideal_part(const StageParams<R>& p
 #pragma unroll
     for (int i = 0; i < 3; ++i) a.m[i] = a.M[i].hi;
   } else {
-    const R itn = R(1) / tn;
+    const R itn = (R)p.tau_dev->inv_taus_new;
     a.e = Tv[0] * itn;
 #pragma unroll
     for (int i = 0; i < 3; ++i) a.m[i] = Tv[1 + i] * itn;
@@ -368,8 +368,10 @@ __device__ __forceinline__ bool correct_root(const EosView<float>& eos, const ff
 template <typename R>
 __device__ __forceinline__ void regulate_shear(R e, R P, R* pi) {
   const R r = visc_ramp(e);
+  if (sizeof(R) == 4 || r != R(1)) {   // FP64: 1 in most cells, and ten products on the narrow pipe
 #pragma unroll
-  for (int q = 0; q < 10; ++q) pi[q] *= r;
+    for (int q = 0; q < 10; ++q) pi[q] *= r;
+  }
   if (r == R(0)) return;
   const R pp = pi[0] * pi[0] - R(2) * (pi[1] * pi[1] + pi[2] * pi[2] + pi[3] * pi[3]) + pi[4] * pi[4] +
                pi[7] * pi[7] + pi[9] * pi[9] + R(2) * (pi[5] * pi[5] + pi[6] * pi[6] + pi[8] * pi[8]);
@@ -650,7 +652,7 @@ __global__ void __launch_bounds__(kBlock) stage_kernel(const StageParams<R> p) {
 #pragma unroll
       for (int m = 0; m < 4; ++m) pi4[m] = pinew[m];
     }
-    const IdealPart<R, VISC> ip = ideal_part<R, VISC>(p, Tnew, Tnl, pi4, (R)p.tau_dev->taus_new);
+    const IdealPart<R, VISC> ip = ideal_part<R, VISC>(p, Tnew, Tnl, pi4);
     const R E = ip.e, Mx = ip.m[0], My = ip.m[1], Me = ip.m[2];
     R en = R(0), ux = R(0), uy = R(0), ue = R(0);
     R Pb = p.Pib ? p.Pib[c] : R(0);   // bulk pressure of the stage's output
@@ -769,7 +771,6 @@ __global__ void __launch_bounds__(kBlock, RecoverMinBlocks<R, GUESS>::value) rec
   R my_e = R(0);
   int my_iters = 0, my_solved = 0, my_polish_iters = 0;
   bool f_rescaled = false, f_fail = false, f_polished = false, f_nonfinite = false, f_nonconv = false;
-  const R tn = (R)p.tau_dev->taus_new;
   // the ideal part E, M of the new T~ (FP32 path: unrounded float-floats for
   // the correction step, their high parts for the FP32 solve)
   double T0v = 0.0;
@@ -787,7 +788,7 @@ __global__ void __launch_bounds__(kBlock, RecoverMinBlocks<R, GUESS>::value) rec
       for (int m = 0; m < 4; ++m) pi4[m] = p.piout[m][c];
     }
     T0v = (double)Tv[0] + (double)Tlv[0];
-    ip = ideal_part<R, VISC>(p, Tv, Tlv, pi4, tn);
+    ip = ideal_part<R, VISC>(p, Tv, Tlv, pi4);
   }
   const R E = ip.e, Mx = ip.m[0], My = ip.m[1], Me = ip.m[2];
   // initial guess for |v|
@@ -842,7 +843,9 @@ __global__ void __launch_bounds__(kBlock, RecoverMinBlocks<R, GUESS>::value) rec
     if (active) {
       const R a = p.pr.u[0][c], b = p.pr.u[1][c], d = p.pr.u[2][c];
       const R w2 = a * a + b * b + d * d;
-      vg = sqrt(w2 / (R(1) + w2));   // |v| of the stage velocity
+      // |v| of the stage velocity (a start: FP32 is enough, off the FP64 pipe)
+      const float f2 = (float)w2;
+      vg = (R)sqrtf(f2 / (1.0f + f2));
     }
   }
   if (active) {
@@ -924,7 +927,7 @@ __global__ void __launch_bounds__(kBlock, RecoverMinBlocks<R, GUESS>::value) rec
     my_T0 = T0v;
     my_e = en;
   }
-  if (p.tau_next && c == 0) store_tau(p.tau_next, p.tau_dev->tau + p.dtau_d, p.tau_dev->inv_end, p.dtau_d, p.inv_deta, p.cartesian);
+  if (p.tau_next && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) store_tau(p.tau_next, p.tau_dev->tau + p.dtau_d, p.tau_dev->inv_end, p.dtau_d, p.inv_deta, p.cartesian);
   const unsigned full = 0xffffffffu;
   const unsigned b_res = __ballot_sync(full, f_rescaled);
   const unsigned b_fail = __ballot_sync(full, f_fail);
