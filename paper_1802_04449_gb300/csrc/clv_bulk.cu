@@ -36,7 +36,7 @@ struct BulkCell {
 };
 
 template <typename R>
-__device__ __forceinline__ BulkCell<R> bulk_cell(const StageParams<R>& p, const R* __restrict__ Pin, long long s,
+__device__ __forceinline__ BulkCell<R> bulk_cell(const StageParams<R>& p, const R* Pin, long long s,
                                                  int axis) {
   const R ux = p.pr.u[0][s], uy = p.pr.u[1][s], ue = p.pr.u[2][s];
   R ut, iu;
@@ -61,7 +61,7 @@ __device__ __forceinline__ R bulk_flux(const BulkCell<R>& a, const BulkCell<R>& 
 }
 
 template <typename R, int STAGE>
-__global__ void __launch_bounds__(kBlock) bulk_stage_kernel(const StageParams<R> p, const R* __restrict__ Pin,
+__global__ void __launch_bounds__(kBlock) bulk_stage_kernel(const StageParams<R> p, const R* Pin,
                                                             const R* Pn, R* Pout,   // Pn == Pout in stage 2
                                                             const R inv_5zs_hbarc) {
   release_next_kernel();

@@ -24,7 +24,7 @@ struct ChargeCell {
 };
 
 template <typename R>
-__device__ __forceinline__ ChargeCell<R> charge_cell(const StageParams<R>& p, const R* __restrict__ Nin, long long s,
+__device__ __forceinline__ ChargeCell<R> charge_cell(const StageParams<R>& p, const R* Nin, long long s,
                                                      int axis) {
   const R ux = p.pr.u[0][s], uy = p.pr.u[1][s], ue = p.pr.u[2][s];
   R ut, iu;
@@ -46,7 +46,7 @@ __device__ __forceinline__ R charge_flux(const ChargeCell<R>& a, const ChargeCel
 }
 
 template <typename R, int STAGE>
-__global__ void __launch_bounds__(kBlock) charge_stage_kernel(const StageParams<R> p, const R* __restrict__ Nin,
+__global__ void __launch_bounds__(kBlock) charge_stage_kernel(const StageParams<R> p, const R* Nin,
                                                               const R* Nn, R* Nout) {   // Nn == Nout in stage 2
   release_next_kernel();
   enter_step_kernel();

@@ -137,7 +137,8 @@ template <typename R> struct StageParams {
 // kGuessMlpAll: the network seeds every cell.
 // Kernels of a step start while their predecessor drains (programmatic
 // dependent launch): nothing of one is done before its predecessor is complete
-// and its writes visible (enter_step_kernel), and the next one may be placed
+// and its writes visible (enter_step_kernel; so what the chain writes is read by
+// plain loads, not through the read-only path), and the next one may be placed
 // once every CTA of this one has released it or is done.  Kernels of many small
 // blocks release it as they start; the stage kernels, at most one wave of large
 // CTAs, do not: the small blocks of the next kernel would be placed on the SMs
@@ -184,7 +185,6 @@ __device__ __forceinline__ void split_index(long long c, int n, long long& row, 
   }
 }
 
-template <typename R> __device__ __forceinline__ R ldg(const R* p) { return __ldg(p); }
 
 template <typename R> struct SolveTraits;
 template <> struct SolveTraits<float> {
@@ -506,11 +506,11 @@ __global__ void __launch_bounds__(kBlock) stage_kernel(const StageParams<R> p) {
       R ut[5], va[5], cs[5];
 #pragma unroll
       for (int d = 0; d < 5; ++d) {
-        const R ux = ldg(p.pr.u[0] + id[d]), uy = ldg(p.pr.u[1] + id[d]), ue = ldg(p.pr.u[2] + id[d]);
+        const R ux = p.pr.u[0][id[d]], uy = p.pr.u[1][id[d]], ue = p.pr.u[2][id[d]];
         ut[d] = sqrt(R(1) + ux * ux + uy * uy + ue * ue);
         const R ua = ax == 1 ? ux : (ax == 2 ? uy : ue);
         va[d] = ua / ut[d];
-        cs[d] = ldg(p.pr.cs + id[d]);
+        cs[d] = p.pr.cs[id[d]];
         if (d == 1 || d == 3) {
           const int side = d == 3 ? 1 : 0;
           unb[ax - 1][side][0] = ut[d];
@@ -526,11 +526,11 @@ __global__ void __launch_bounds__(kBlock) stage_kernel(const StageParams<R> p) {
         R v[5];
 #pragma unroll
         for (int d = 0; d < 5; ++d) {
-          if (q < 4) v[d] = ldg(p.T[q] + id[d]);
-          else if (VISC && q < 14) v[d] = ldg(p.pi[q - 4] + id[d]);
+          if (q < 4) v[d] = p.T[q][id[d]];
+          else if (VISC && q < 14) v[d] = p.pi[q - 4][id[d]];
           else if (q == IU) v[d] = ut[d];
           else if (q == IV) v[d] = va[d];
-          else v[d] = ldg(p.pr.P + id[d]);
+          else v[d] = p.pr.P[id[d]];
         }
         const R s1 = minmod(v[2] - v[1], v[1] - v[0]);
         const R s2 = minmod(v[2] - v[1], v[3] - v[2]);
