@@ -1411,9 +1411,10 @@ clv_status clv_mlp_loss_grad(const float* d_params, const float* d_X, const floa
   if (s != CLV_OK) return s;
   cudaStream_t st = (cudaStream_t)stream;
   const int blocks = mlp_grad_blocks(n);
-  mlp_grad_kernel<<<blocks, kMlpGradThreads, mlp_grad_smem_bytes(), st>>>(d_params, d_X, d_Y, n, n, 0ull, 0, d_work);
-  mlp_reduce_kernel<<<(kMlpPartialRow + 31) / 32, 32 * kMlpReduceGroups, 0, st>>>(d_work, blocks, d_grad, d_loss,
-                                                                                  MlpAdam{});
+  launch_step_kernel(mlp_grad_kernel, blocks, kMlpGradThreads, mlp_grad_smem_bytes(), st, d_params, d_X, d_Y, n, n, 0ull,
+                     0, d_work);
+  launch_step_kernel(mlp_reduce_kernel, (kMlpPartialRow + 31) / 32, 32 * kMlpReduceGroups, 0, st, d_work, blocks, d_grad,
+                     d_loss, MlpAdam{});
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? CLV_OK : fail(nullptr, CLV_ECUDA, cudaGetErrorString(e));
 }
@@ -1431,10 +1432,10 @@ clv_status clv_mlp_train(float* d_params, float* d_work, const float* d_X, const
   float* partial = d_work + 3 * kMlpParams;
   const int blocks = mlp_grad_blocks(batch);
   for (int it = 0; it < iters; ++it) {
-    mlp_grad_kernel<<<blocks, kMlpGradThreads, mlp_grad_smem_bytes(), st>>>(d_params, d_X, d_Y, n, batch, seed,
-                                                                           step0 + it, partial);
-    mlp_reduce_kernel<<<(kMlpPartialRow + 31) / 32, 32 * kMlpReduceGroups, 0, st>>>(
-        partial, blocks, g, d_loss + it, MlpAdam{d_params, m, v, step0 + it + 1, lr});
+    launch_step_kernel(mlp_grad_kernel, blocks, kMlpGradThreads, mlp_grad_smem_bytes(), st, d_params, d_X, d_Y, n, batch,
+                       seed, step0 + it, partial);
+    launch_step_kernel(mlp_reduce_kernel, (kMlpPartialRow + 31) / 32, 32 * kMlpReduceGroups, 0, st, partial, blocks, g,
+                       d_loss + it, MlpAdam{d_params, m, v, step0 + it + 1, lr});
   }
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? CLV_OK : fail(nullptr, CLV_ECUDA, cudaGetErrorString(e));

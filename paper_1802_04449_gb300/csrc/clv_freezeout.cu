@@ -21,6 +21,7 @@
 #include <string>
 
 #include "clv.h"
+#include "clv_launch.cuh"
 
 // defined in clv_api.cu: message returned by clv_last_error(NULL)
 void clv_set_global_error(const char* msg);
@@ -64,6 +65,8 @@ __device__ __forceinline__ void decode_cube(unsigned c, int cy, int ce, int& i, 
 template <typename R>
 __global__ void __launch_bounds__(kThreads) fo_classify_kernel(FoArgs<R> a, unsigned char* __restrict__ flags,
                                                                int* __restrict__ counts) {
+  clv::release_next_kernel();
+  clv::enter_step_kernel();
   const long long c = (long long)blockIdx.x * kThreads + threadIdx.x;
   int crossed = 0;
   if (c < a.ncube) {
@@ -79,10 +82,12 @@ __global__ void __launch_bounds__(kThreads) fo_classify_kernel(FoArgs<R> a, unsi
   if (threadIdx.x == 0) counts[blockIdx.x] = n;
 }
 
-__global__ void __launch_bounds__(kScanThreads) fo_scan_kernel(const int* __restrict__ counts, int nblk,
+__global__ void __launch_bounds__(kScanThreads) fo_scan_kernel(const int* counts, int nblk,
                                                                long long* __restrict__ offsets,
                                                                long long* __restrict__ total,
                                                                int64_t* __restrict__ d_count) {
+  clv::release_next_kernel();
+  clv::enter_step_kernel();
   __shared__ long long warp_sum[kScanThreads / 32];
   __shared__ long long carry;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -121,10 +126,12 @@ __global__ void __launch_bounds__(kScanThreads) fo_scan_kernel(const int* __rest
   }
 }
 
-__global__ void __launch_bounds__(kThreads) fo_compact_kernel(const unsigned char* __restrict__ flags,
+__global__ void __launch_bounds__(kThreads) fo_compact_kernel(const unsigned char* flags,
                                                               long long ncube,
-                                                              const long long* __restrict__ offsets,
+                                                              const long long* offsets,
                                                               int* __restrict__ list) {
+  clv::release_next_kernel();
+  clv::enter_step_kernel();
   __shared__ int warp_cnt[kThreads / 32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const long long c = (long long)blockIdx.x * kThreads + threadIdx.x;
@@ -264,10 +271,11 @@ __device__ __forceinline__ R warp_sum(R x) {
 // the warps are latency-bound, and 32 resident warps per SM instead of 24
 // (78 registers) made a find 5% faster.
 template <typename R>
-__global__ void __launch_bounds__(kElemThreads, sizeof(R) == 4 ? 4 : 2) fo_elements_kernel(FoArgs<R> a, const int* __restrict__ list,
-                                                                   const long long* __restrict__ total,
+__global__ void __launch_bounds__(kElemThreads, sizeof(R) == 4 ? 4 : 2) fo_elements_kernel(FoArgs<R> a, const int* list,
+                                                                   const long long* total,
                                                                    long long capacity, R* __restrict__ rec,
                                                                    int64_t* __restrict__ cube_out) {
+  clv::enter_step_kernel();
   const int lane = threadIdx.x & 31;
   // the ordering of the axes of this lane's simplex: lexicographic rank s
   const int s = lane < 24 ? lane : lane - 24;
@@ -297,12 +305,23 @@ __global__ void __launch_bounds__(kElemThreads, sizeof(R) == 4 ? 4 : 2) fo_eleme
   long long n = *total;
   if (n > capacity) n = capacity;
   const long long nwarps = (long long)gridDim.x * (kElemThreads / 32);
-  for (long long e = (long long)blockIdx.x * (kElemThreads / 32) + (threadIdx.x >> 5); e < n; e += nwarps) {
-    const int c = list[e];
+  // the next element's index and corner values are fetched while the current one
+  // is worked on (a warp has few elements and their loads depend on each other)
+  auto corner_value = [&](int cube) {
+    int ci, cj, ck;
+    decode_cube((unsigned)cube, a.cy, a.ce, ci, cj, ck);
+    return lane < 16 ? a.e[lane & 1][corner_offset(a, ci, cj, ck, lane)] - a.ef : R(0);
+  };
+  long long e = (long long)blockIdx.x * (kElemThreads / 32) + (threadIdx.x >> 5);
+  int c = e < n ? list[e] : 0;
+  R fq = e < n ? corner_value(c) : R(0);
+  int c_next = 0;
+  R fq_next = 0;
+  for (; e < n; e += nwarps, c = c_next, fq = fq_next) {
+    const bool more = e + nwarps < n;
+    c_next = more ? list[e + nwarps] : 0;
     int i, j, k;
     decode_cube((unsigned)c, a.cy, a.ce, i, j, k);
-    R fq = 0;
-    if (lane < 16) fq = a.e[lane & 1][corner_offset(a, i, j, k, lane)] - a.ef;
     R f[5];
 #pragma unroll
     for (int m = 0; m < 5; ++m) {
@@ -314,6 +333,7 @@ __global__ void __launch_bounds__(kElemThreads, sizeof(R) == 4 ? 4 : 2) fo_eleme
     for (int m = 0; m < 4; ++m) pc.dS[m] = pc.Ac[m] = 0;
     pc.A = 0;
     if (lane < 24) simplex_piece<R>(a, vpack, f, perm, fs, pc);
+    fq_next = more ? corner_value(c_next) : R(0);
     R dS[4], Ac[4];
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
@@ -474,9 +494,9 @@ clv_status fo_run(const clv_fo_grid* g, const clv_fo_slice* s0, const clv_fo_sli
   long long* offsets = reinterpret_cast<long long*>(sc + L.offsets);
   unsigned char* flags = reinterpret_cast<unsigned char*>(sc + L.flags);
   int* list = reinterpret_cast<int*>(sc + L.list);
-  fo_classify_kernel<R><<<L.nblk, kThreads, 0, st>>>(a, flags, counts);
-  fo_scan_kernel<<<1, kScanThreads, 0, st>>>(counts, L.nblk, offsets, total, d_count);
-  fo_compact_kernel<<<L.nblk, kThreads, 0, st>>>(flags, L.ncube, offsets, list);
+  clv::launch_step_kernel(fo_classify_kernel<R>, L.nblk, kThreads, 0, st, a, flags, counts);
+  clv::launch_step_kernel(fo_scan_kernel, 1, kScanThreads, 0, st, counts, L.nblk, offsets, total, d_count);
+  clv::launch_step_kernel(fo_compact_kernel, L.nblk, kThreads, 0, st, flags, L.ncube, offsets, list);
   int dev = 0, sms = 1, per_sm = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -484,8 +504,8 @@ clv_status fo_run(const clv_fo_grid* g, const clv_fo_slice* s0, const clv_fo_sli
   const long long need = (L.ncube + kElemThreads / 32 - 1) / (kElemThreads / 32);
   long long blocks = (long long)sms * (per_sm > 0 ? per_sm : 1);
   if (blocks > need) blocks = need;
-  fo_elements_kernel<R><<<(unsigned)blocks, kElemThreads, 0, st>>>(a, list, total, (long long)capacity,
-                                                                   static_cast<R*>(d_rec), d_cube);
+  clv::launch_step_kernel(fo_elements_kernel<R>, (unsigned)blocks, kElemThreads, 0, st, a, list, total,
+                          (long long)capacity, static_cast<R*>(d_rec), d_cube);
   const cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) {
     clv_set_global_error((std::string("clv_fo_find: ") + cudaGetErrorString(err)).c_str());

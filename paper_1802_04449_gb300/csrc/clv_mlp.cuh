@@ -14,6 +14,7 @@
 #include <cuda_bf16.h>
 
 #include "clv_device.cuh"
+#include "clv_launch.cuh"
 
 namespace clv {
 
@@ -286,11 +287,13 @@ __device__ __forceinline__ void mlp_scale_tile(const float2 (&a)[4][2], float* D
   }
 }
 
-static __global__ void __launch_bounds__(kMlpGradThreads, 2) mlp_grad_kernel(const float* __restrict__ params,
+static __global__ void __launch_bounds__(kMlpGradThreads, 2) mlp_grad_kernel(const float* params,
                                                                   const float* __restrict__ X,
                                                                   const float* __restrict__ Y, long long n,
                                                                   long long batch, unsigned long long seed, int iter,
                                                                   float* __restrict__ partial) {
+  release_next_kernel();
+  enter_step_kernel();
   extern __shared__ __align__(16) float sm[];
   __shared__ long long s_idx[kMlpChunk];   // sample of each slot of the chunk, -1 past the batch
   __shared__ float s_red[kMlpGradThreads / 32][2];
@@ -481,9 +484,11 @@ struct MlpAdam {
 // kMlpReduceGroups-th row in order (coalesced), and the first warp adds the
 // warps' sums in order.
 constexpr int kMlpReduceGroups = 16;
-static __global__ void __launch_bounds__(32 * kMlpReduceGroups) mlp_reduce_kernel(const float* __restrict__ partial,
+static __global__ void __launch_bounds__(32 * kMlpReduceGroups) mlp_reduce_kernel(const float* partial,
                                                                                  int nblocks, float* grad,
                                                                                  float* loss, const MlpAdam ad) {
+  release_next_kernel();
+  enter_step_kernel();
   __shared__ float s[kMlpReduceGroups][33];
   const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
   const int p = blockIdx.x * 32 + lane;
