@@ -375,7 +375,10 @@ __device__ __forceinline__ RootResult solve_primitive(const EosView<R>& q, C eps
     // an FP32 lookup no longer sees a step of eps below its rounding: P is
     // constant there, and the step that takes it so lands on the root
     if constexpr (sizeof(CE) < sizeof(C))
-      if (fabs(M * dv) <= C(6e-8) * e) dv = -Ops::div(g, den);
+      if (fabs(M * dv) <= C(6e-8) * e) {
+        dv = -Ops::div(g, den);
+        if (CE(E - M * (v + dv)) == CE(e)) { v += dv; ok = true; break; }   // the same lookup: this is its root
+      }
     // converged when the Newton step is below tol; otherwise keep the iterate
     // strictly inside the shrinking bracket
     if (fabs(dv) <= tol) { v += dv; ok = true; break; }

@@ -481,12 +481,14 @@ __device__ __forceinline__ void stage_tile_body(const StageParams<R>& p, const E
               un[1] = cb[CI::UN * ncell]; un[2] = cb[(CI::UN + 1) * ncell]; un[3] = cb[(CI::UN + 2) * ncell];
               un[0] = sqrt(R(1) + un[1] * un[1] + un[2] * un[2] + un[3] * un[3]);
             }
-            R ustar0 = un[0];
+            R ustar0 = un[0], iustar0 = R(0);   // iustar0: 1/u*^tau (FP64)
             if constexpr (VISC) {
               const R us1 = R(2) * un[1] - cb[CI::UP * ncell];
               const R us2 = R(2) * un[2] - cb[(CI::UP + 1) * ncell];
               const R us3 = R(2) * un[3] - cb[(CI::UP + 2) * ncell];
-              ustar0 = sqrt(R(1) + us1 * us1 + us2 * us2 + us3 * us3);
+              const R us = R(1) + us1 * us1 + us2 * us2 + us3 * us3;
+              if constexpr (F64) sqrt_and_inverse(us, ustar0, iustar0);
+              else ustar0 = sqrt(us);
               R ul[4];
               if constexpr (STAGE == 1) {
                 ul[0] = ustar0; ul[1] = us1; ul[2] = us2; ul[3] = us3;
@@ -536,7 +538,7 @@ __device__ __forceinline__ void stage_tile_body(const StageParams<R>& p, const E
                 }
               }
               if constexpr (VISC) {
-                const R inv = R(1) / ustar0, cn = un[0] * inv, ch = hh * inv;
+                const R inv = F64 ? iustar0 : R(1) / ustar0, cn = un[0] * inv, ch = hh * inv;
 #pragma unroll
                 for (int r = 0; r < 10; ++r) pinew[r] = cn * W0[4 + r] + ch * S[4 + r];
                 regulate_shear<R>(e, Pe, pinew);
