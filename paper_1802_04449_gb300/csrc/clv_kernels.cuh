@@ -359,7 +359,7 @@ __device__ __forceinline__ void regulate_shear(R e, R P, R* pi) {
 }
 
 // Israel-Stewart source (Sec. 2, Eq. pimn with lambda_2 = lambda_3 = 0):
-// du[a][b] = d~_a u~^b.
+// du[a][b] = d~_a u~^b, added to S.
 template <typename R>
 __device__ __forceinline__ void shear_source(R geo, const R u[4], R du[4][4], const R pi[10], R e,
                                              R P, R inv_taupi, const IsCoef<R>& is, R* S) {
@@ -393,7 +393,7 @@ __device__ __forceinline__ void shear_source(R geo, const R u[4], R du[4][4], co
       const R sm = R(metric_sign(m)), sn = R(metric_sign(n));
       R d = sm * du[m][n] + sn * du[n][m];
       if (m == n) d -= sm * th23;
-      S[q] = ep5 * d + u[m] * C[n] + u[n] * C[m] - decay * pi[q];
+      S[q] = S[q] + ep5 * d + u[m] * C[n] + u[n] * C[m] - decay * pi[q];
     }
   // -(lambda_1 / tau_pi) pi^<mu_l pi^nu>l in tilde components: Y = pi g~ pi,
   // X = Delta^m_a Delta^n_c Y^ac - Delta^mn (Delta_ac Y^ac) / 3
@@ -575,10 +575,7 @@ __global__ void __launch_bounds__(kBlock) stage_kernel(const StageParams<R> p) {
       R Tc, c2dummy;
       eos_eval<R, R>(p.eos, e, Pe, Tc, c2dummy);
       const R inv_taupi = Tc * p.is.inv_b_etas_hbarc;
-      R Spi[10];
-      shear_source<R>(ts.geo, u, du, pic, e, Pe, inv_taupi, p.is, Spi);
-#pragma unroll
-      for (int q = 0; q < 10; ++q) S[4 + q] += Spi[q];
+      shear_source<R>(ts.geo, u, du, pic, e, Pe, inv_taupi, p.is, S + 4);
     }
     // ---------------- stage update (Sec. 3) ----------------
     // FP32 path: the increment h S added exactly to the float-float T~

@@ -514,12 +514,10 @@ __device__ __forceinline__ void stage_tile_body(const StageParams<R>& p, const E
               R Tc, c2d;
               eos_eval<R, R>(p.eos, e, Pe, Tc, c2d);
               const R inv_taupi = Tc * ev.is.inv_b_etas_hbarc;
-              R pic[10], Spi[10];
+              R pic[10];
 #pragma unroll
               for (int r = 0; r < 10; ++r) pic[r] = W0[4 + r];
-              shear_source<R>(ts.geo, u, du, pic, e, Pe, inv_taupi, ev.is, Spi);
-#pragma unroll
-              for (int r = 0; r < 10; ++r) S[4 + r] += Spi[r];
+              shear_source<R>(ts.geo, u, du, pic, e, Pe, inv_taupi, ev.is, S + 4);
             }
             // ---- stage update (Sec. 3).  FP32 path: T~ is a float-float
             // pair (high part staged in W0, low part prefetched) and the
