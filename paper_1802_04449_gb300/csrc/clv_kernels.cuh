@@ -390,6 +390,14 @@ __device__ __forceinline__ void shear_source(R geo, const R u[4], R du[4][4], co
 #pragma unroll
     for (int n = m; n < 4; ++n) {
       const int q = sym_index(m, n);
+      if (q == 0) {
+        // in a slow cell the theta terms of sigma^{00} leave (1 - u0^2) theta,
+        // of order v^2: gathered, they round as theta / 3 each (pi^{00} of
+        // spots at rest moved by 3e-5 after 5 steps)
+        const R sigma = R(2) * du[0][0] - R(2) * u[0] * Du[0] - R(2.0 / 3.0) * (R(1) - u[0] * u[0]) * theta;
+        S[0] = S[0] + (ep5 * sigma - R(2) * u[0] * w[0] - decay * pi[0]);
+        continue;
+      }
       const R sm = R(metric_sign(m)), sn = R(metric_sign(n));
       R d = sm * du[m][n] + sn * du[n][m];
       if (m == n) d -= sm * th23;
