@@ -401,7 +401,12 @@ __device__ __forceinline__ void shear_source(R geo, const R u[4], R du[4][4], co
       const R sm = R(metric_sign(m)), sn = R(metric_sign(n));
       R d = sm * du[m][n] + sn * du[n][m];
       if (m == n) d -= sm * th23;
-      S[q] = S[q] + ep5 * d + u[m] * C[n] + u[n] * C[m] - decay * pi[q];
+      // FP32: terms that cancel are summed before the larger flux sum is added
+      // (420 steps of 97 x 97 x 41 cells against the oracle: 2.7e-5 to 5.2e-5
+      // over the guesses, 3.7e-5 to 1.3e-4 added one by one).  FP64: one by
+      // one, 0.7% faster there
+      if constexpr (sizeof(R) == 8) S[q] = S[q] + ep5 * d + u[m] * C[n] + u[n] * C[m] - decay * pi[q];
+      else S[q] = S[q] + (ep5 * d + u[m] * C[n] + u[n] * C[m] - decay * pi[q]);
     }
   // -(lambda_1 / tau_pi) pi^<mu_l pi^nu>l in tilde components: Y = pi g~ pi,
   // X = Delta^m_a Delta^n_c Y^ac - Delta^mn (Delta_ac Y^ac) / 3
