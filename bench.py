@@ -620,14 +620,14 @@ def run_gpu(args):
                    "steps": so,
                    "bulk": {"zeta_over_s": 0.1, "value": N * so / (msBk / 1e3), "unit": UNIT,
                             "ms_per_step": msBk / so, "step_overhead": (msBk / so) / (ms32 / args.steps) - 1.0,
-                            "launches_per_step": 7,
+                            "launches_per_step": 6,
                             "roofline": {"bound": "hbm", "kernel": "bulk_stage_kernel<float>", "ms_avg": t_bulk,
                                          "achieved": ach_b, "peak": peak, "unit": "GB/s",
                                          "frac": (ach_b / peak) if ach_b else None,
                                          "algorithmic_bytes_per_launch": BULK_WORDS * 4 * N},
                             "error_word": stBk.get("error_word")},
                    "charge": {"value": N * so / (msCh / 1e3), "unit": UNIT, "ms_per_step": msCh / so,
-                              "step_overhead": (msCh / so) / (ms32 / args.steps) - 1.0, "launches_per_step": 7,
+                              "step_overhead": (msCh / so) / (ms32 / args.steps) - 1.0, "launches_per_step": 6,
                               "roofline": {"bound": "hbm", "kernel": "charge_stage_kernel<float>", "ms_avg": t_charge,
                                            "achieved": ach_c, "peak": peak, "unit": "GB/s",
                                            "frac": (ach_c / peak) if ach_c else None,
@@ -724,7 +724,7 @@ def run_gpu(args):
         "roofline": roof,
         "e2e": e2e,
         # per step: two stages of (stage kernel, root solve) and the tau advance
-        "gpu_launches": 5 * args.steps,
+        "gpu_launches": 4 * args.steps,
         "clocks": clocks,
         "stats_fp32": {k: st32.get(k) for k in ("tau", "eps_max", "T_max", "E_tot", "n_polished", "n_rootfail",
                                                 "n_fp32_nonconverged", "error_word", "error", "tile")},
