@@ -620,7 +620,7 @@ def run_gpu(args):
                    "steps": so,
                    "bulk": {"zeta_over_s": 0.1, "value": N * so / (msBk / 1e3), "unit": UNIT,
                             "ms_per_step": msBk / so, "step_overhead": (msBk / so) / (ms32 / args.steps) - 1.0,
-                            "launches_per_step": 6,
+                           "launches_per_step": 6,
                             "roofline": {"bound": "hbm", "kernel": "bulk_stage_kernel<float>", "ms_avg": t_bulk,
                                          "achieved": ach_b, "peak": peak, "unit": "GB/s",
                                          "frac": (ach_b / peak) if ach_b else None,
@@ -723,7 +723,7 @@ def run_gpu(args):
         "cooperfrye": cooperfrye,
         "roofline": roof,
         "e2e": e2e,
-        # per step: two stages of (stage kernel, root solve) and the tau advance
+        # per step: two stages of (stage kernel, root solve); the last one advances tau
         "gpu_launches": 4 * args.steps,
         "clocks": clocks,
         "stats_fp32": {k: st32.get(k) for k in ("tau", "eps_max", "T_max", "E_tot", "n_polished", "n_rootfail",
