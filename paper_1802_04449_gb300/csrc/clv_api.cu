@@ -1088,17 +1088,7 @@ __global__ void __launch_bounds__(kBlock) prims_from_T_kernel(double* a0, double
     atomicOr(err, 2u);
     e = ux = uy = ue = 0.0;
   } else {
-    // single-precision handle: the FP64 solve starts from the FP32 root (two
-    // or three steps on the FP64 pipe instead of six)
-    double v0 = -1.0;
-    if constexpr (sizeof(R) == 4) {
-      float ef, a, b, d, vf = -1.0f;
-      solve_primitive<float, float>(eos, (float)eps_cut, (float)E, (float)Mx, (float)My, (float)Me,
-                                    SolveTraits<float>::tol, SolveTraits<float>::maxit, ef, a, b, d, &vf);
-      v0 = (double)vf;
-    }
-    const RootResult rr =
-        solve_primitive<double, R, R>(eos, eps_cut, E, Mx, My, Me, 1e-15, 200, e, ux, uy, ue, &v0);
+    const RootResult rr = solve_primitive<double, R, R>(eos, eps_cut, E, Mx, My, Me, 1e-15, 200, e, ux, uy, ue);
     if (rr.rescaled) atomicAdd(counters + 0, 1ull);
     if (rr.iters < 0) { atomicAdd(counters + 1, 1ull); atomicOr(err, 1u); }
   }

@@ -39,10 +39,10 @@ template <typename R>
 __device__ __forceinline__ BulkCell<R> bulk_cell(const StageParams<R>& p, const R* Pin, long long s,
                                                  int axis) {
   const R ux = p.pr.u[0][s], uy = p.pr.u[1][s], ue = p.pr.u[2][s];
-  R ut, iu;
-  sqrt_and_inverse(R(1) + ux * ux + uy * uy + ue * ue, ut, iu);
   const R ua = axis == 0 ? ux : (axis == 1 ? uy : ue);
-  return BulkCell<R>{ut, ua * iu, Pin[s], p.pr.cs[s], ua};
+  R ut, v;
+  ut_and_v(ux, uy, ue, ua, ut, v);
+  return BulkCell<R>{ut, v, Pin[s], p.pr.cs[s], ua};
 }
 
 // flux v^a u~^tau Pi at the interface between cells b and c from cells a, b, c, d

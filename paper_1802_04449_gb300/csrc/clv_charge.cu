@@ -27,10 +27,10 @@ template <typename R>
 __device__ __forceinline__ ChargeCell<R> charge_cell(const StageParams<R>& p, const R* Nin, long long s,
                                                      int axis) {
   const R ux = p.pr.u[0][s], uy = p.pr.u[1][s], ue = p.pr.u[2][s];
-  R ut, iu;
-  sqrt_and_inverse(R(1) + ux * ux + uy * uy + ue * ue, ut, iu);
   const R ua = axis == 0 ? ux : (axis == 1 ? uy : ue);
-  return ChargeCell<R>{Nin[s], ua * iu, p.pr.cs[s]};
+  R ut, v;
+  ut_and_v(ux, uy, ue, ua, ut, v);
+  return ChargeCell<R>{Nin[s], v, p.pr.cs[s]};
 }
 
 // flux at the interface between cells b and c from cells a, b, c, d

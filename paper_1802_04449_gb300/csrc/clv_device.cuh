@@ -312,10 +312,11 @@ __device__ __forceinline__ RootResult solve_primitive(const EosView<R>& q, C eps
   C P, cs2, dPde;   // dPde: d(P + Pshift)/d eps, 0 on the floor (cs2 keeps the table's value)
   C v;
   bool fixed = FIXED;
-  // conformal EOS: f is a quadratic in v (off the pressure floor), and its root
-  // is the start, which the first Newton step then confirms
+  // conformal EOS in FP64: f is a quadratic in v (off the pressure floor), and
+  // its root is the start, which the first Newton step then confirms.  (FP32
+  // starts from the guess: another start ends on another rounding of the root.)
   C vconf = C(-1);
-  if (!FIXED && q.kind == 0) {
+  if (sizeof(CE) == 8 && !FIXED && q.kind == 0) {
     const C A = C(4.0 / 3.0) * E + Pshift, disc = A * A - C(4.0 / 3.0) * (M * M);
     if (A > C(0) && disc > C(0)) vconf = Ops::div(C(2) * M, A + Ops::sqrt_(disc));
   }
@@ -371,14 +372,7 @@ __device__ __forceinline__ RootResult solve_primitive(const EosView<R>& q, C eps
     const C den = E + P;
     const C g = v * den - M;
     if (g > C(0)) hi = v; else lo = v;
-    C dv = -Ops::div(den * g, den * den - dPde * (M * M));
-    // an FP32 lookup no longer sees a step of eps below its rounding: P is
-    // constant there, and the step that takes it so lands on the root
-    if constexpr (sizeof(CE) < sizeof(C))
-      if (fabs(M * dv) <= C(6e-8) * e) {
-        dv = -Ops::div(g, den);
-        if (CE(E - M * (v + dv)) == CE(e)) { v += dv; ok = true; break; }   // the same lookup: this is its root
-      }
+    const C dv = -Ops::div(den * g, den * den - dPde * (M * M));
     // converged when the Newton step is below tol; otherwise keep the iterate
     // strictly inside the shrinking bracket
     if (fabs(dv) <= tol) { v += dv; ok = true; break; }
@@ -489,20 +483,33 @@ __device__ __forceinline__ void cp_async_wait_prior() { asm volatile("cp.async.w
 // differences of equal products cancel exactly.
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+// Product and sum rounded once.
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
 
-__device__ __forceinline__ void sqrt_and_inverse(float a, float& root, float& inv) {
-  inv = rsqrtf(a);
-  const float r = mul_rn(a, inv);
-  root = fmaf(fmaf(-r, r, a), 0.5f * inv, r);
+// u~^tau of a cell and the velocity ua/u~^tau (FP64: one root and no division)
+__device__ __forceinline__ void ut_and_v(double ux, double uy, double ue, double ua, double& ut, double& v) {
+  double inv;
+  sqrt_and_inverse(1.0 + ux * ux + uy * uy + ue * ue, ut, inv);
+  v = ua * inv;
+}
+__device__ __forceinline__ void ut_and_v(float ux, float uy, float ue, float ua, float& ut, float& v) {
+  ut = sqrt(1.0f + ux * ux + uy * uy + ue * ue);
+  v = ua / ut;
 }
 
-// max of (|v| + c_s)/(1 + |v| c_s) of two sides, the larger found by
-// cross-multiplication: one division
-template <typename R> __device__ __forceinline__ R signal_speed(R vl, R csl, R vr, R csr) {
-  const R al = fabs(vl), ar = fabs(vr);
-  const R nl = al + csl, dl = R(1) + al * csl, nr = ar + csr, dr = R(1) + ar * csr;
+// max of (|v| + c_s)/(1 + |v| c_s) of two sides.  FP64: the larger found by
+// cross-multiplication, one division.  FP32: that of the rounded quotients
+// (near a tie the other way is an ulp off, which the shear source amplifies).
+__device__ __forceinline__ double signal_speed(double vl, double csl, double vr, double csr) {
+  const double al = fabs(vl), ar = fabs(vr);
+  const double nl = al + csl, dl = 1.0 + al * csl, nr = ar + csr, dr = 1.0 + ar * csr;
   const bool rs = nr * dl > nl * dr;
   return (rs ? nr : nl) / (rs ? dr : dl);
+}
+__device__ __forceinline__ float signal_speed(float vl, float csl, float vr, float csr) {
+  const float al = fabs(vl), ar = fabs(vr);
+  return fmax((al + csl) / (1.0f + al * csl), (ar + csr) / (1.0f + ar * csr));
 }
 
 // minmod(a, b): 0 unless a and b share a sign, else the one of smaller

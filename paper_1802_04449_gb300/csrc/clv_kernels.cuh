@@ -163,11 +163,6 @@ __device__ __forceinline__ void split_index(long long c, int n, long long& row, 
 template <typename R> struct SolveTraits;
 template <> struct SolveTraits<float> {
   static constexpr float tol = 5e-7f;
-  // last step of a solve that a further Newton step follows: below v = 0.99
-  // the step's error is 0.5 |dv|^2 or less plus |dv| times the mismatch of
-  // the tabulated c_s^2 and the table's slope (1e-3): 2e-8 at 2e-5, under the
-  // 1e-7 of the FP32 residual that ends either solve
-  static constexpr float tol_corrected = 2e-5f;
   static constexpr int maxit = 40;
 };
 template <> struct SolveTraits<double> {
@@ -358,56 +353,14 @@ __device__ __forceinline__ void regulate_shear(R e, R P, R* pi) {
   }
 }
 
-// Israel-Stewart source (Sec. 2, Eq. pimn with lambda_2 = lambda_3 = 0):
-// du[a][b] = d~_a u~^b, added to S.
+// Products that round on their own (shear_source): the direct kernel, and stage 1 of the tiled one
+constexpr int kApartDirect = 7, kApartTile1 = 6;
+
+// The parts of the shear source beyond sigma and the decay: lambda_1 and the
+// Christoffel terms.
 template <typename R>
-__device__ __forceinline__ void shear_source(R geo, const R u[4], R du[4][4], const R pi[10], R e,
-                                             R P, R inv_taupi, const IsCoef<R>& is, R* S) {
-  // corrected tilde covariant derivatives (Eq. dtuz)
-  du[3][0] += geo * u[3];
-  du[3][3] += geo * u[0];
-  const R theta = du[0][0] + du[1][1] + du[2][2] + du[3][3];
-  R Du[4];
-#pragma unroll
-  for (int b = 0; b < 4; ++b) Du[b] = u[0] * du[0][b] + u[1] * du[1][b] + u[2] * du[2][b] + u[3] * du[3][b];
-  // w^m = g~_{bb} pi~^{m b} Du^b
-  R w[4];
-#pragma unroll
-  for (int m = 0; m < 4; ++m)
-    w[m] = pi[sym_index(m, 0)] * Du[0] - pi[sym_index(m, 1)] * Du[1] - pi[sym_index(m, 2)] * Du[2] -
-           pi[sym_index(m, 3)] * Du[3];
-  const R ep5 = (e + P) * is.inv_b;
-  const R decay = inv_taupi + theta * R(1.0 / 3.0) + geo * u[0];
-  // ep5 sigma^{mn} - (u^m w^n + u^n w^m) with sigma^{mn} = g^m d_m u^n + g^n
-  // d_n u^m - u^m Du^n - u^n Du^m - (2/3) (g^{mn} - u^m u^n) theta, gathered
-  // as ep5 (...) + u^m C^n + u^n C^m, C^m = ep5 (theta u^m / 3 - Du^m) - w^m
-  const R th23 = R(2.0 / 3.0) * theta;
-  R C[4];
-#pragma unroll
-  for (int m = 0; m < 4; ++m) C[m] = ep5 * (R(0.5) * th23 * u[m] - Du[m]) - w[m];
-#pragma unroll
-  for (int m = 0; m < 4; ++m)
-#pragma unroll
-    for (int n = m; n < 4; ++n) {
-      const int q = sym_index(m, n);
-      if (q == 0) {
-        // in a slow cell the theta terms of sigma^{00} leave (1 - u0^2) theta,
-        // of order v^2: gathered, they round as theta / 3 each (pi^{00} of
-        // spots at rest moved by 3e-5 after 5 steps)
-        const R sigma = R(2) * du[0][0] - R(2) * u[0] * Du[0] - R(2.0 / 3.0) * (R(1) - u[0] * u[0]) * theta;
-        S[0] = S[0] + (ep5 * sigma - R(2) * u[0] * w[0] - decay * pi[0]);
-        continue;
-      }
-      const R sm = R(metric_sign(m)), sn = R(metric_sign(n));
-      R d = sm * du[m][n] + sn * du[n][m];
-      if (m == n) d -= sm * th23;
-      // FP32: terms that cancel are summed before the larger flux sum is added
-      // (420 steps of 97 x 97 x 41 cells against the oracle: 2.7e-5 to 5.2e-5
-      // over the guesses, 3.7e-5 to 1.3e-4 added one by one).  FP64: one by
-      // one, 0.7% faster there
-      if constexpr (sizeof(R) == 8) S[q] = S[q] + ep5 * d + u[m] * C[n] + u[n] * C[m] - decay * pi[q];
-      else S[q] = S[q] + (ep5 * d + u[m] * C[n] + u[n] * C[m] - decay * pi[q]);
-    }
+__device__ __forceinline__ void shear_source_rest(R geo, const R u[4], const R pi[10], R e, R inv_taupi,
+                                                  const IsCoef<R>& is, R* S) {
   // -(lambda_1 / tau_pi) pi^<mu_l pi^nu>l in tilde components: Y = pi g~ pi,
   // X = Delta^m_a Delta^n_c Y^ac - Delta^mn (Delta_ac Y^ac) / 3
   if (is.lambda1_hat != R(0) && e > R(0)) {
@@ -441,13 +394,134 @@ __device__ __forceinline__ void shear_source(R geo, const R u[4], R du[4][4], co
   }
   // Christoffel terms I^{mu nu} (Eq. Ipi), with a minus sign in S_pi
   const R gu = geo * u[3];
-  S[0] -= R(2) * gu * pi[3];
-  S[1] -= gu * pi[6];
-  S[2] -= gu * pi[8];
-  S[3] -= gu * (pi[0] + pi[9]);
-  S[6] -= gu * pi[1];
-  S[8] -= gu * pi[2];
-  S[9] -= R(2) * gu * pi[3];
+  S[0] = fma_rn(-R(2) * gu, pi[3], S[0]);
+  S[1] = fma_rn(-gu, pi[6], S[1]);
+  S[2] = fma_rn(-gu, pi[8], S[2]);
+  S[3] = fma_rn(-gu, pi[0] + pi[9], S[3]);
+  S[6] = fma_rn(-gu, pi[1], S[6]);
+  S[8] = fma_rn(-gu, pi[2], S[8]);
+  S[9] = fma_rn(-R(2) * gu, pi[3], S[9]);
+}
+
+// Israel-Stewart source (Sec. 2, Eq. pimn with lambda_2 = lambda_3 = 0):
+// du[a][b] = d~_a u~^b, added to S.
+template <int APART>
+__device__ __forceinline__ void shear_source(double geo, const double u[4], double du[4][4], const double pi[10],
+                                             double e, double P, double inv_taupi, const IsCoef<double>& is,
+                                             double* S) {
+  using R = double;
+  // corrected tilde covariant derivatives (Eq. dtuz)
+  du[3][0] += geo * u[3];
+  du[3][3] += geo * u[0];
+  const R theta = du[0][0] + du[1][1] + du[2][2] + du[3][3];
+  R Du[4];
+#pragma unroll
+  for (int b = 0; b < 4; ++b) Du[b] = u[0] * du[0][b] + u[1] * du[1][b] + u[2] * du[2][b] + u[3] * du[3][b];
+  // w^m = g~_{bb} pi~^{m b} Du^b
+  R w[4];
+#pragma unroll
+  for (int m = 0; m < 4; ++m)
+    w[m] = pi[sym_index(m, 0)] * Du[0] - pi[sym_index(m, 1)] * Du[1] - pi[sym_index(m, 2)] * Du[2] -
+           pi[sym_index(m, 3)] * Du[3];
+  const R ep5 = (e + P) * is.inv_b;
+  const R decay = inv_taupi + theta * R(1.0 / 3.0) + geo * u[0];
+  // ep5 sigma^{mn} - (u^m w^n + u^n w^m) with sigma^{mn} = g^m d_m u^n + g^n
+  // d_n u^m - u^m Du^n - u^n Du^m - (2/3) (g^{mn} - u^m u^n) theta, gathered
+  // as ep5 (...) + u^m C^n + u^n C^m, C^m = ep5 (theta u^m / 3 - Du^m) - w^m
+  const R th23 = R(2.0 / 3.0) * theta;
+  R C[4];
+#pragma unroll
+  for (int m = 0; m < 4; ++m) C[m] = ep5 * (R(0.5) * th23 * u[m] - Du[m]) - w[m];
+#pragma unroll
+  for (int m = 0; m < 4; ++m)
+#pragma unroll
+    for (int n = m; n < 4; ++n) {
+      const int q = sym_index(m, n);
+      if (q == 0) {
+        // in a slow cell the theta terms of sigma^{00} leave (1 - u0^2) theta,
+        // of order v^2: gathered, they round as theta / 3 each
+        const R sigma = R(2) * du[0][0] - R(2) * u[0] * Du[0] - R(2.0 / 3.0) * (R(1) - u[0] * u[0]) * theta;
+        S[0] = S[0] + (ep5 * sigma - R(2) * u[0] * w[0] - decay * pi[0]);
+        continue;
+      }
+      const R sm = R(metric_sign(m)), sn = R(metric_sign(n));
+      R d = sm * du[m][n] + sn * du[n][m];
+      if (m == n) d -= sm * th23;
+      S[q] = S[q] + ep5 * d + u[m] * C[n] + u[n] * C[m] - decay * pi[q];
+    }
+  shear_source_rest<R>(geo, u, pi, e, inv_taupi, is, S);
+}
+
+// The same in FP32, where the order of the operations and every rounding are
+// part of the result.  In a boosted cell of a dilute fringe (gamma 5 to 8) the
+// time derivative of u~^tau, a difference of nearly equal numbers, enters
+// pi~^{00} times gamma^2: one rounding more or less, here or in the velocities
+// that this reads, moved pi~^{00} by 1e-4 to 8e-4 of its largest value in six
+// steps (261 x 261 x 121 cells, mini-jet start).  So each multiply-add is
+// written out and none is left for the compiler to form, which it did in
+// another way in each kernel.  APART keeps what the three kernels had: bit m,
+// the product u~^m u~^m of sigma^{mm} is rounded before it is subtracted, and
+// with any bit so is u~^eta / tau.  The gathered sum of FP64 would be 1% faster
+// (20 steps of 97 x 97 x 41 cells: 3.85 ms against 3.89).
+template <int APART>
+__device__ __forceinline__ void shear_source(float geo, const float u[4], float du[4][4], const float pi[10], float e,
+                                             float P, float inv_taupi, const IsCoef<float>& is, float* S) {
+  du[3][0] = APART ? __fadd_rn(du[3][0], __fmul_rn(geo, u[3])) : __fmaf_rn(geo, u[3], du[3][0]);
+  du[3][3] = __fmaf_rn(geo, u[0], du[3][3]);
+  const float theta = __fadd_rn(__fadd_rn(__fadd_rn(du[0][0], du[1][1]), du[2][2]), du[3][3]);
+  float Du[4], w[4];
+#pragma unroll
+  for (int b = 0; b < 4; ++b)
+    Du[b] = __fmaf_rn(u[3], du[3][b],
+                      __fmaf_rn(u[2], du[2][b], __fmaf_rn(u[0], du[0][b], __fmul_rn(u[1], du[1][b]))));
+#pragma unroll
+  for (int m = 0; m < 4; ++m)
+    w[m] = __fmaf_rn(-pi[sym_index(m, 3)], Du[3],
+                     __fmaf_rn(-pi[sym_index(m, 2)], Du[2],
+                               __fmaf_rn(pi[sym_index(m, 0)], Du[0], -__fmul_rn(pi[sym_index(m, 1)], Du[1]))));
+  const float ep5 = __fmul_rn(__fadd_rn(e, P), is.inv_b);
+  const float decay = __fmaf_rn(geo, u[0], __fmaf_rn(theta, 1.0f / 3.0f, inv_taupi));
+  float s[10];
+#pragma unroll
+  for (int m = 0; m < 4; ++m)
+#pragma unroll
+    for (int n = m; n < 4; ++n) {
+      const int q = sym_index(m, n);
+      // sigma^{mn} = g^m d_m u^n + g^n d_n u^m - u^m Du^n - u^n Du^m - (2/3) (g^{mn} - u^m u^n) theta
+      float g = m == n ? (float)metric_sign(m) : 0.0f;
+      if (m == n && (APART >> m & 1)) g = __fsub_rn(g, __fmul_rn(u[m], u[n]));
+      else g = __fmaf_rn(-u[m], u[n], g);
+      float sigma = __fadd_rn((float)metric_sign(m) * du[m][n], (float)metric_sign(n) * du[n][m]);
+      sigma = __fmaf_rn(-u[n], Du[m], __fmaf_rn(-u[m], Du[n], sigma));
+      sigma = __fmaf_rn(-__fmul_rn(2.0f / 3.0f, g), theta, sigma);
+      s[q] = __fsub_rn(__fmaf_rn(ep5, sigma, -__fmul_rn(decay, pi[q])),
+                       __fmaf_rn(u[m], w[n], __fmul_rn(u[n], w[m])));
+    }
+  shear_source_rest<float>(geo, u, pi, e, inv_taupi, is, s);
+#pragma unroll
+  for (int q = 0; q < 10; ++q) S[q] = __fadd_rn(S[q], s[q]);
+}
+
+// pi~ after a stage: (un pin [+ us pi] + h S) inv, the second term in stage 2.
+// FP64 takes the factor inv into the coefficients; FP32 with its roundings
+// written out, as in the source.
+template <int STAGE>
+__device__ __forceinline__ void shear_update(double inv, double un, const double pin[10], double us,
+                                             const double pi[10], double h, const double* S, double pinew[10]) {
+  const double cn = un * inv, cs = us * inv, ch = h * inv;
+#pragma unroll
+  for (int q = 0; q < 10; ++q)
+    pinew[q] = STAGE == 1 ? cn * pin[q] + ch * S[q] : cn * pin[q] + cs * pi[q] + ch * S[q];
+}
+template <int STAGE>
+__device__ __forceinline__ void shear_update(float inv, float un, const float pin[10], float us, const float pi[10],
+                                             float h, const float* S, float pinew[10]) {
+#pragma unroll
+  for (int q = 0; q < 10; ++q) {
+    const float a = STAGE == 1 ? __fmaf_rn(un, pin[q], __fmul_rn(h, S[q]))
+                               : __fmaf_rn(h, S[q], __fmaf_rn(un, pin[q], __fmul_rn(us, pi[q])));
+    pinew[q] = __fmul_rn(a, inv);
+  }
 }
 
 template <typename R, int STAGE, bool VISC, bool STATS>
@@ -588,7 +662,7 @@ __global__ void __launch_bounds__(kBlock) stage_kernel(const StageParams<R> p) {
       R Tc, c2dummy;
       eos_eval<R, R>(p.eos, e, Pe, Tc, c2dummy);
       const R inv_taupi = Tc * p.is.inv_b_etas_hbarc;
-      shear_source<R>(ts.geo, u, du, pic, e, Pe, inv_taupi, p.is, S + 4);
+      shear_source<kApartDirect>(ts.geo, u, du, pic, e, Pe, inv_taupi, p.is, S + 4);
     }
     // ---------------- stage update (Sec. 3) ----------------
     // FP32 path: the increment h S added exactly to the float-float T~
@@ -607,9 +681,7 @@ __global__ void __launch_bounds__(kBlock) stage_kernel(const StageParams<R> p) {
         }
       }
       if constexpr (VISC) {
-        const R inv = R(1) / ustar0, cn = un[0] * inv, ch = h * inv;
-#pragma unroll
-        for (int q = 0; q < 10; ++q) pinew[q] = cn * pic[q] + ch * S[4 + q];
+        shear_update<1>(R(1) / ustar0, un[0], pic, R(0), pic, h, S + 4, pinew);
         regulate_shear<R>(e, Pe, pinew);
       }
     } else {
@@ -624,9 +696,10 @@ __global__ void __launch_bounds__(kBlock) stage_kernel(const StageParams<R> p) {
         }
       }
       if constexpr (VISC) {
-        const R inv = R(0.5) / u[0], cn = un[0] * inv, cs = ustar0 * inv, ch = h * inv;
+        R pin[10];
 #pragma unroll
-        for (int q = 0; q < 10; ++q) pinew[q] = cn * p.pin[q][c] + cs * pic[q] + ch * S[4 + q];
+        for (int q = 0; q < 10; ++q) pin[q] = p.pin[q][c];
+        shear_update<2>(R(0.5) / u[0], un[0], pin, ustar0, pic, h, S + 4, pinew);
         regulate_shear<R>(e, Pe, pinew);
       }
     }
@@ -839,15 +912,8 @@ __global__ void __launch_bounds__(kBlock, RecoverMinBlocks<R, GUESS>::value) rec
     if (!(isfinite(E) && isfinite(Mx) && isfinite(My) && isfinite(Me))) {
       f_nonfinite = true;
     } else {
-      // FP32: a cell below the velocity threshold of the FP64 refinement gets
-      // a Newton step of its own below (correct_root, or the refinement near
-      // the cut), which takes a root known to tol_corrected to the same
-      // result as one known to tol
-      R tol = SolveTraits<R>::tol;
-      if constexpr (sizeof(R) == 4)
-        if (Mx * Mx + My * My + Me * Me <= (p.polish_v * E) * (p.polish_v * E)) tol = SolveTraits<R>::tol_corrected;
-      RootResult rr = solve_primitive<R, R>(p.eos, p.eps_cut, E, Mx, My, Me, tol, SolveTraits<R>::maxit, en, ux, uy,
-                                            ue, &vg, &at_root, Pb);
+      RootResult rr = solve_primitive<R, R>(p.eos, p.eps_cut, E, Mx, My, Me, SolveTraits<R>::tol,
+                                            SolveTraits<R>::maxit, en, ux, uy, ue, &vg, &at_root, Pb);
       f_rescaled = rr.rescaled;
       my_iters = rr.iters > 0 ? rr.iters : 0;
       my_solved = rr.iters > 0 ? 1 : 0;

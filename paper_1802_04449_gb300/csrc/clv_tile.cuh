@@ -517,7 +517,7 @@ __device__ __forceinline__ void stage_tile_body(const StageParams<R>& p, const E
               R pic[10];
 #pragma unroll
               for (int r = 0; r < 10; ++r) pic[r] = W0[4 + r];
-              shear_source<R>(ts.geo, u, du, pic, e, Pe, inv_taupi, ev.is, S + 4);
+              shear_source<STAGE == 1 && !BATCH ? kApartTile1 : 0>(ts.geo, u, du, pic, e, Pe, inv_taupi, ev.is, S + 4);
             }
             // ---- stage update (Sec. 3).  FP32 path: T~ is a float-float
             // pair (high part staged in W0, low part prefetched) and the
@@ -536,9 +536,7 @@ __device__ __forceinline__ void stage_tile_body(const StageParams<R>& p, const E
                 }
               }
               if constexpr (VISC) {
-                const R inv = F64 ? iustar0 : R(1) / ustar0, cn = un[0] * inv, ch = hh * inv;
-#pragma unroll
-                for (int r = 0; r < 10; ++r) pinew[r] = cn * W0[4 + r] + ch * S[4 + r];
+                shear_update<1>(F64 ? iustar0 : R(1) / ustar0, un[0], W0 + 4, R(0), W0 + 4, hh, S + 4, pinew);
                 regulate_shear<R>(e, Pe, pinew);
               }
             } else {
@@ -555,10 +553,10 @@ __device__ __forceinline__ void stage_tile_body(const StageParams<R>& p, const E
                 }
               }
               if constexpr (VISC) {
-                const R inv = R(0.5) / u[0], cn = un[0] * inv, cs = ustar0 * inv, ch = hh * inv;
+                R pin[10];
 #pragma unroll
-                for (int r = 0; r < 10; ++r)
-                  pinew[r] = cn * cb[(CI::PIN + r) * ncell] + cs * W0[4 + r] + ch * S[4 + r];
+                for (int r = 0; r < 10; ++r) pin[r] = cb[(CI::PIN + r) * ncell];
+                shear_update<2>(R(0.5) / u[0], un[0], pin, ustar0, W0 + 4, hh, S + 4, pinew);
                 regulate_shear<R>(e, Pe, pinew);
               }
             }
