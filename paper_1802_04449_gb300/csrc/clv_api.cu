@@ -911,10 +911,15 @@ template <typename R> clv_status finish_initial(clv_handle* h) {
   return initial_end<R>(h);
 }
 
+// in_stage: the arrays `in` lie in the stage-2 shear buffers.  These return to
+// zeros before the first-step predictor runs: its T~ goes there, and their
+// padding slots, which no stage writes but the root solve reads, are vacuum.
 template <typename R>
-clv_status set_initial_impl(clv_handle* h, const double* const in[4], const double* pi, bool host) {
+clv_status set_initial_impl(clv_handle* h, const double* const in[4], const double* pi, bool host,
+                            bool in_stage = false) {
   h->initial_pi = pi && h->viscous;
   clv_status s = load_initial_range<R>(h, 0, h->N, h->Nc, h->cfg.neta, h->nep, h->viscous, in, pi, host);
+  if (s == CLV_OK && in_stage) CLV_CUDA(h, clear_stage_shear(h));
   return s != CLV_OK ? s : finish_initial<R>(h);
 }
 
@@ -1122,18 +1127,16 @@ static clv_status set_initial_T_any(clv_handle* h, const double* T, bool host) {
   unsigned err = 0;
   CLV_CUDA(h, cudaMemcpyAsync(&err, &h->dstats->err, 4, cudaMemcpyDeviceToHost, h->stream));
   CLV_CUDA(h, cudaStreamSynchronize(h->stream));
-  if (err & 2u) return fail(h, CLV_ENONFINITE, "non-finite T^{tau mu} in the initial state");
-  if (err & 1u) return fail(h, CLV_EROOT, "root solve of the initial state hit its iteration cap");
+  if (err) {
+    CLV_CUDA(h, clear_stage_shear(h));
+    if (err & 2u) return fail(h, CLV_ENONFINITE, "non-finite T^{tau mu} in the initial state");
+    return fail(h, CLV_EROOT, "root solve of the initial state hit its iteration cap");
+  }
   const double* in[4] = {a, a + N, a + 2 * N, a + 3 * N};
   h->cur = 0;
   h->prev = 1;
-  clv_status st =
-      h->rsize == 8 ? set_initial_impl<double>(h, in, nullptr, false) : set_initial_impl<float>(h, in, nullptr, false);
-  if (st != CLV_OK) return st;
-  // the scratch is consumed (stream order): the stage buffers return to zeros, as the
-  // padding slots of the eta rows, which the stages never write, must stay vacuum
-  CLV_CUDA(h, clear_stage_shear(h));
-  return CLV_OK;
+  return h->rsize == 8 ? set_initial_impl<double>(h, in, nullptr, false, true)
+                       : set_initial_impl<float>(h, in, nullptr, false, true);
 }
 
 static clv_status set_initial_any(clv_handle* h, const double* eps, const double* ux, const double* uy,

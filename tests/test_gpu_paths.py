@@ -104,3 +104,24 @@ def test_initial_T_is_kept_by_the_predictor(prec, tol):
     for k, want in (("Tty", case.tau0 * w * np.sqrt(ut2) * f["uy"]), ("Tte", case.tau0 * w * np.sqrt(ut2) * f["ueta"]),
                     ("Ttt", case.tau0 * (w * ut2 - P))):
         assert np.all(np.abs(f[k] - want)[live] <= tol * 50 * np.abs(f["Ttt"])[live]), k
+
+
+@pytest.mark.parametrize("refused", [False, True])
+@pytest.mark.parametrize("prec", [clv.CLV_FP64, clv.CLV_FP32])
+def test_padding_stays_vacuum_through_an_initial_T(prec, refused):
+    """Rows of 9 cells have a pitch of 12: in a checkpoint taken before the first step the padding of T~ and pi~ is 0 and that of
+    the previous step's primitives equals that of the current ones, vacuum -- also after an initial T that was refused."""
+    case = I.hotspot_event(nx=15, ny=13, neta=9, n_spots=30, seed=2, eta_over_s=0.08)
+    h = clv.from_case(case, prec)
+    T = np.stack([case.eps, 0.3 * case.eps, -0.2 * case.eps, 0.1 * case.eps])
+    if refused:
+        with pytest.raises(clv.ClvError):
+            h.set_initial_T(np.where(np.arange(9) == 4, np.nan, T))
+        h.set_initial(case.eps, case.ux, case.uy, case.ueta)
+    else:
+        h.set_initial_T(T)
+    R = np.float64 if prec == clv.CLV_FP64 else np.float32
+    f = np.frombuffer(bytes(h.get_state()), R, offset=88).reshape(-1, 15, 13, 12)[..., 9:]
+    assert len(f) == (26 if prec == clv.CLV_FP64 else 30)
+    assert np.all(f[:-12] == 0) and np.all(f[-12:-8] == 0)
+    assert np.array_equal(f[-6:], f[-12:-6])
