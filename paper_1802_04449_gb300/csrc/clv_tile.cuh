@@ -304,8 +304,9 @@ __device__ __forceinline__ void stage_tile_body(const StageParams<R>& p, const E
   // tile with its halo (no corners), the two planes on either side of the
   // chunk only the tile's own columns (their x-stencil); vectors without any
   // are not copied, and only these cells are converted to v, which costs a
-  // square root and a division each.  (A thread has at most one vector:
-  // (TJ + 4) box_width(TK) / 4 <= 256 for up to 256 positions.)
+  // square root and a division each.  (A thread has one vector, or two in
+  // long tiles of one or two columns: (TJ + 4) box_width(TK) / 4 <= 264 for up
+  // to 256 positions.  Bits 4 to 7 are the second one's.)
   unsigned need_out = 0, need_own = 0;
   for (int w = w0, sh = 0; w < vend; w += nthr, sh += 4) {
     const int bj = (4 * w) / BW, c0 = kb0 + 4 * w - bj * BW;

@@ -125,3 +125,23 @@ def test_padding_stays_vacuum_through_an_initial_T(prec, refused):
     assert len(f) == (26 if prec == clv.CLV_FP64 else 30)
     assert np.all(f[:-12] == 0) and np.all(f[-12:-8] == 0)
     assert np.array_equal(f[-6:], f[-12:-6])
+
+
+@pytest.mark.parametrize("shape", [(81, 2), (82, 2), (84, 2), (124, 1), (125, 1), (127, 1)])
+def test_long_tiles_whose_threads_stage_two_vectors(shape):
+    """FP64 tiles of one or two columns have up to 264 four-cell vectors in a plane for 256 threads (81 x 2 and 124 x 1 are the
+    last with one or none for each).  Fields agree with the default tile's bit for bit."""
+    case = I.hotspot_event(nx=7, ny=129, neta=5, n_spots=60, seed=6, eta_over_s=0.0)
+
+    def run(tile):
+        g = clv.from_case(case, clv.CLV_FP64)
+        g.set_initial(case.eps, case.ux, case.uy, case.ueta)
+        if tile:
+            g.set_tile(*tile, 0)
+            assert g.tile()["TJ"] == tile[0]
+        g.step(3)
+        return g.get(FIELDS[:5])
+
+    ref, got = run(None), run(shape)
+    for k in ref:
+        assert np.array_equal(got[k], ref[k]), k
