@@ -145,3 +145,27 @@ def test_long_tiles_whose_threads_stage_two_vectors(shape):
     ref, got = run(None), run(shape)
     for k in ref:
         assert np.array_equal(got[k], ref[k]), k
+
+def test_logarithm_of_the_fp64_lookup():
+    """P(eps) of the table on both sides of the edges and in the middle of the 64 intervals of the mantissa that the logarithm
+    is tabulated over, for every binary exponent of the table, read back through T~^{tau x} = tau (eps + P) u~^tau u~^x.
+
+    Tolerance: P varies by at most d ln P / d ln eps < 2 times an error of ln eps.  ln eps - ln eps_0 < 26 is rounded three
+    times here and there, 26 x 6 x 1.1e-16 = 1.7e-14; with T~ and the division by u~ (3 x 1.1e-16 of eps + P < 12 P): 4e-14."""
+    eos = I.crossover_eos()
+    lne0, dlne, n = eos["lne0"], eos["dlne"], len(eos["P"])
+    edge = 1 + np.arange(64) / 64
+    m = np.concatenate([edge, np.nextafter(edge, 0), np.nextafter(edge, 2), edge + 1 / 128])
+    e = (m[None] * 2.0 ** np.arange(-22, 13)[:, None]).ravel()
+    e = e[(e > np.exp(lne0) * 1.01) & (e < np.exp(lne0 + (n - 1) * dlne) * 0.99)]
+    e = e[:len(e) // 4 * 4]
+    shape = (len(e) // 4, 2, 2)
+    x = (np.log(e) - lne0) / dlne
+    k = np.clip(np.floor(x), 0, n - 2).astype(int)
+    P = eos["P"][k] + (x - k) * (eos["P"][k + 1] - eos["P"][k])
+    assert np.all(e / P < 11) and np.max(np.diff(np.log(eos["P"])) / dlne) < 2
+    h = clv.Hydro(*shape, 0.2, 0.2, 0.2, 1.0, 0.01, 0.0, eos, clv.CLV_FP64)
+    z = np.zeros(shape)
+    h.set_initial(e.reshape(shape), z + 0.75, z, z)   # u~^tau = 1.25
+    got = h.get(["Ttx"])["Ttx"].ravel() / (1.25 * 0.75) - e
+    assert np.all(np.abs(got - P) <= 4e-14 * P), float(np.max(np.abs(got - P) / P))
