@@ -620,7 +620,7 @@ def run_gpu(args):
                    "steps": so,
                    "bulk": {"zeta_over_s": 0.1, "value": N * so / (msBk / 1e3), "unit": UNIT,
                             "ms_per_step": msBk / so, "step_overhead": (msBk / so) / (ms32 / args.steps) - 1.0,
-                           "launches_per_step": 6,
+                            "launches_per_step": 6,
                             "roofline": {"bound": "hbm", "kernel": "bulk_stage_kernel<float>", "ms_avg": t_bulk,
                                          "achieved": ach_b, "peak": peak, "unit": "GB/s",
                                          "frac": (ach_b / peak) if ach_b else None,

@@ -292,12 +292,14 @@ clv_status clv_mlp_train(float* d_params, float* d_work, const float* d_X, const
  * (CLV_EINVAL).  The batch starts (first-step predictor) at the first
  * clv_step, after every event's initial state was set.
  * Each event's tile follows a tiling policy shared by the batch: at most
- * max_threads threads per CTA (the shape with the least modelled cost) and x
- * chunks of about `chunk` planes; the default is 384 (128 in FP64) threads and
- * the chunk whose work items end soonest in the model.  The persistent stage launch holds as
- * many CTAs per SM as the device's occupancy calculator allows for the
- * policy's largest tile.  clv_autotune on a started batch
- * times the current policy and up to max_candidates others (thread caps of
+ * max_threads interface positions (TJ + 1)(TK + 1) per tile (the shape with
+ * the least modelled cost) and x chunks of about `chunk` planes; the default
+ * is 384 (128 in FP64) positions and the chunk whose work items end soonest in
+ * the model.  A CTA has a thread per position in FP32, always 256 threads in
+ * FP64.  The persistent stage launch holds as many CTAs per SM as the device's
+ * occupancy calculator allows for the policy's largest tile.  clv_autotune on
+ * a started batch
+ * times the current policy and up to max_candidates others (position caps of
  * 1, 3/4 and 1/2 of the limit, chunks of 16-64 planes; reps stage-1 launches
  * each, which leave the state unchanged), keeps the fastest (the current
  * unless another is at least 2% faster) and reports it in clv_tile_info as
@@ -319,8 +321,8 @@ clv_status clv_batch_get_fields(clv_handle* h, int event, uint32_t which_mask, d
  * Synchronises the stream. */
 clv_status clv_batch_event_stats(clv_handle* h, int event, clv_stats* out);
 
-/* Explicit tiling policy of a batch (see above): max_threads in [32, 384]
- * (capped at 128 in FP64), chunk in [1, 4096] planes.  CLV_EINVAL if out of
+/* Explicit tiling policy of a batch (see above): max_threads, the interface
+ * positions of a tile, in [32, 384] (capped at 128 in FP64), chunk in [1, 4096] planes.  CLV_EINVAL if out of
  * range, not a batch, or if a tile would exceed the shared memory of a CTA.
  * Synchronises the stream. */
 clv_status clv_batch_set_schedule(clv_handle* h, int max_threads, int chunk);
@@ -372,22 +374,26 @@ clv_status clv_set_graphs(clv_handle* h, int enable);
 
 /* ---------------- tile shape of the stage kernel ----------------
  * The stage kernel works on (y, eta_s) tiles of TJ x TK cells, each CTA
- * marching along x over CX planes ((TJ + 1)(TK + 1) threads per CTA).  The
- * shape changes no result, only the speed. */
+ * marching along x over CX planes.  A tile has (TJ + 1)(TK + 1) interface
+ * positions: a thread for each in FP32, while an FP64 CTA always has 256
+ * threads.  The shape changes no result, only the speed. */
 typedef struct {
   int TJ, TK, CX;            /* tile rows (y), columns (eta_s), planes per CTA (x) */
-  int threads;               /* threads per CTA */
+  int threads;               /* interface positions (TJ + 1)(TK + 1): in FP32 the threads of a CTA
+                                (FP64: 256 threads); a batch: those of its largest tile */
   int blocks;                /* CTAs per stage launch */
-  int smem_bytes;            /* dynamic shared memory per CTA */
+  int smem_bytes;            /* dynamic shared memory per CTA (a grid of at most one CTA per SM asks
+                                for more than half an SM's, so that no two share one) */
   double ms;                 /* clv_autotune: mean stage-1 time of the chosen shape (ms) */
 } clv_tile_info;
 
 clv_status clv_get_tile(clv_handle* h, clv_tile_info* out);
 
 /* Explicit shape; CX = 0 picks the x chunking by the makespan rule (with as
- * many CTAs per SM as the occupancy calculator allows at this shape).
- * CLV_EINVAL if out of range or beyond the thread limit ((TJ + 1)(TK + 1) <=
- * 384 in FP32, 128 in FP64) or the 227 KiB shared-memory limit of a CTA. */
+ * many CTAs per SM as this shape's shared memory and the registers of the
+ * stage kernel, 168 a thread in FP32 and 256 in FP64, leave room for).
+ * CLV_EINVAL if out of range or beyond the limit of positions ((TJ + 1)(TK + 1)
+ * <= 384 in FP32, 256 in FP64) or the 227 KiB shared-memory limit of a CTA. */
 clv_status clv_set_tile(clv_handle* h, int TJ, int TK, int CX);
 
 /* Autotuner: times the current shape and up to max_candidates modelled-best

@@ -30,19 +30,9 @@ template <typename R> struct IsCoef {
   R lambda1_hat;
 };
 
-// T~^{tau mu} keeps ~48 significant bits on the FP32 path: a float-float pair
-// T~ = T + Tl (high parts T, low parts Tl, both float arrays).  It is the
-// conserved energy-momentum that every stage accumulates into; in the dilute,
-// fast-moving edge of an event the rest-frame density eps = E - M v is a
-// small difference of its components (E/eps ~ gamma^2), so plain FP32
-// storage of T~ turned its rounding into percent-level errors of eps there
-// after a few hundred steps.  The stencil reads the high parts (fluxes and
-// sources stay FP32); the update adds the FP32 increment to the pair exactly,
-// and the recovery forms E and M from the pair.  The FP64 path stores T~ in
-// T and leaves Tl unused.
 // tau of a step and what its kernels take from it: 1/tau of its end (tau +
 // dtau; 1 in Cartesian mode) as a float-float pair for the FP32 recovery, and
-// per stage the tau factors of TauS in both precisions.  One thread forms them
+// per stage the tau factors in both precisions.  One thread forms them
 // per step: formed by every thread of a kernel, their FP64 divisions alone took
 // the FP64 pipe (2 lanes an SM and cycle) 18 us on 97 x 97 x 41 cells and 2 us
 // of every CTA of a stage.  A handle has two slots, used by alternate steps
@@ -81,6 +71,16 @@ __device__ __forceinline__ void store_tau(TauSlot* s, double tau, double it, dou
   }
 }
 
+// T~^{tau mu} keeps ~48 significant bits on the FP32 path: a float-float pair
+// T~ = T + Tl (high parts T, low parts Tl, both float arrays).  It is the
+// conserved energy-momentum that every stage accumulates into; in the dilute,
+// fast-moving edge of an event the rest-frame density eps = E - M v is a
+// small difference of its components (E/eps ~ gamma^2), so plain FP32
+// storage of T~ turned its rounding into percent-level errors of eps there
+// after a few hundred steps.  The stencil reads the high parts (fluxes and
+// sources stay FP32); the update adds the FP32 increment to the pair exactly,
+// and the recovery forms E and M from the pair.  The FP64 path stores T~ in
+// T and leaves Tl unused.
 template <typename R> struct StageParams {
   // fields of the stage being differentiated (stage 1: step n, stage 2: stage-1 result)
   const R* T[4];
@@ -103,9 +103,9 @@ template <typename R> struct StageParams {
   int nep;     // eta pitch of the layout (ne rounded up to a multiple of 4)
   int xhalo;   // 1: x planes -2, -1, nx, nx + 1 are stored halo planes (an x-slab); no clamping in x
   long long N;
-  // tau of the step lives on the device (advanced by a kernel after every
-  // step), so the launches of a step do not depend on it and a captured step
-  // replays unchanged
+  // tau of the step lives on the device (the last root solve of a step writes
+  // the next one's), so the launches of a step do not depend on it and a
+  // captured step replays unchanged
   const TauSlot* tau_dev;
   TauSlot* tau_next;   // stage 2: tau of the next step, written by the root solve (nullptr in stage 1)
   double dtau_d;
@@ -809,8 +809,8 @@ __global__ void __launch_bounds__(kBlock) stage_kernel(const StageParams<R> p) {
 // from the stage velocity, writes P and c_s, zeroes pi~ in vacuum cells, and
 // (STATS) reduces sum T~^{tau tau} and max eps.
 // blocks of 256 threads (or as many smaller ones) per SM: the dependent table
-// lookups of the root solve need the occupancy.  In FP32 six, with 42 registers
-// and a small spill, are 10% faster than four (261 x 261 x 121 cells: 239 -> 213
+// lookups of the root solve need the occupancy.  In FP32 six, with 40 registers
+// and a spill of 64 to 116 bytes, are 10% faster than four (261 x 261 x 121 cells: 239 -> 213
 // us a launch); with the network, which then spills more, four are best
 template <typename R, int GUESS>
 struct RecoverMinBlocks {

@@ -6,10 +6,10 @@
 //      memory as the per-cell reconstruction fields (T~, pi~, u~^tau, v, P, c_s),
 //      by cp.async one plane ahead, together with the per-cell inputs of the
 //      cell that plane's iteration outputs;
-//   2. every y- and eta_s-interface flux of the tile is computed once: the
-//      block has (TJ+1) x (TK+1) threads, thread (a, b) computes the
-//      y-interface below row a of column b and the eta_s-interface left of
-//      column b of row a, so each thread does at most one interface per axis;
+//   2. every y- and eta_s-interface flux of the tile is computed once.  FP32:
+//      the block has a thread for each of the tile's (TJ+1)(TK+1) interface
+//      positions, and a thread does at most one interface per axis; FP64: a
+//      block of 256 threads takes the interfaces as tasks;
 //   3. each cell thread forms its y/eta_s flux differences and the y/eta_s
 //      derivatives of u~, which wait in shared memory for two planes.
 // The x-direction stencil lives in a register window over the thread's own
