@@ -257,9 +257,7 @@ __global__ void cf_reduce_kernel(const double* __restrict__ partial, int nchunk,
 
 // ---- host side
 
-// CTAs of the sum that the chip holds at a time: five per SM in FP32 (94
-// registers), three in FP64
-constexpr long long kResidentF32 = 152 * 5, kResidentF64 = 152 * 3;
+constexpr int kTargetCtas = 1216;   // momentum tiles x element chunks x species, about 8 per SM
 
 struct Plan {
   long long npts, nthr;
@@ -276,18 +274,10 @@ Plan make_plan(long long nel, int nsp, int nY, int npt, int nphi, size_t rs) {
   P.nthr = (long long)nY * npt * ((nphi + kPhi - 1) / kPhi);
   P.gx = (int)((P.nthr + kThreads - 1) / kThreads);
   const long long tiles = (nel + kTile - 1) / kTile;
-  // chunks for the fewest tiles in a row: waves of CTAs x (tiles of a chunk + a
-  // third of one for its start), the fewer chunks within 2%.  60,000 elements on
-  // 3 x 41 x 15 x 48 points: 17 chunks in two full waves, 3.52 ms; 14 chunks, which
-  // fill 1.6 waves, 3.58
-  const long long ctas = (long long)P.gx * nsp, slots = rs == 8 ? kResidentF64 : kResidentF32;
-  const long long most = 64 + 2 * slots / ctas;
-  long long want = tiles > 0 ? 1 : 0;
-  double best = 1e300;
-  for (long long n = 1; n <= tiles && n <= most; ++n) {
-    const double cost = (double)((ctas * n + slots - 1) / slots) * ((double)((tiles + n - 1) / n) + 0.33);
-    if (cost < 0.98 * best) { best = cost; want = n; }
-  }
+  long long want = (kTargetCtas + (long long)P.gx * nsp - 1) / ((long long)P.gx * nsp);
+  if (want < 1) want = 1;
+  if (want > tiles) want = tiles;
+  if (want > 65535) want = 65535;
   const long long tiles_per_chunk = want > 0 ? (tiles + want - 1) / want : 0;
   P.chunk = tiles_per_chunk * kTile;
   P.nchunk = P.chunk > 0 ? (int)((nel + P.chunk - 1) / P.chunk) : 0;
