@@ -955,7 +955,10 @@ clv_status export_fields(clv_handle* h, const int* which, int nf, double* dst, l
     field_source<R>(h, which[i], off, x.hi[m], x.lo[m]);
     x.dst[m++] = d;
   }
-  if (m) export_kernel<R><<<dim3(transfer_grid(n), (unsigned)m), kBlock, 0, h->stream>>>(x, n, ne, nep);
+  if (m && n * m <= kTransferSmall)
+    export_kernel<R, 1><<<dim3(grid_of(n), (unsigned)m), kBlock, 0, h->stream>>>(x, n, ne, nep);
+  else if (m)
+    export_kernel<R, kTransfer><<<dim3(transfer_grid(n), (unsigned)m), kBlock, 0, h->stream>>>(x, n, ne, nep);
   CLV_CUDA(h, cudaGetLastError());
   return CLV_OK;
 }

@@ -1213,16 +1213,21 @@ template <typename R> struct ExportSet {
 };
 // Cells of a thread in the initial-state and export transfers: loads in flight
 // for the bandwidth.  Export of 18 fields of 261 x 261 x 121 cells: 0.80 ms
-// with one converted by the FP64 pipe.
+// with one converted by the FP64 pipe.  An export of no more values than the
+// chip has threads for four times takes one cell a thread: the launch is its
+// time (four fields of 65 x 63 x 31 cells to the host 105 -> 100 us), and with
+// four cells half of the SMs have no block; beyond that four are faster (one
+// field of 160 x 160 x 80 cells 12.9 -> 10.8 us).
 constexpr int kTransfer = 4;
+constexpr long long kTransferSmall = 4ll * 152 * 2048;
 
-template <typename R>
+template <typename R, int PER>
 __global__ void __launch_bounds__(kBlock) export_kernel(const ExportSet<R> x, long long N, int ne, int nep) {
   const R *hi = x.hi[blockIdx.y], *lo = x.lo[blockIdx.y];
   double* dst = x.dst[blockIdx.y];
 #pragma unroll
-  for (int i = 0; i < kTransfer; ++i) {
-    const long long c = ((long long)blockIdx.x * kTransfer + i) * kBlock + threadIdx.x;
+  for (int i = 0; i < PER; ++i) {
+    const long long c = ((long long)blockIdx.x * PER + i) * kBlock + threadIdx.x;
     if (c >= N) return;
     const long long k = padded_index(c, ne, nep);
     double v = widen(hi[k]);

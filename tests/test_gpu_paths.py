@@ -169,3 +169,22 @@ def test_logarithm_of_the_fp64_lookup():
     h.set_initial(e.reshape(shape), z + 0.75, z, z)   # u~^tau = 1.25
     got = h.get(["Ttx"])["Ttx"].ravel() / (1.25 * 0.75) - e
     assert np.all(np.abs(got - P) <= 4e-14 * P), float(np.max(np.abs(got - P) / P))
+
+
+@pytest.mark.parametrize("prec", [clv.CLV_FP64, clv.CLV_FP32])
+@pytest.mark.parametrize("shape", [(152, 128, 64), (151, 131, 63)])
+def test_exports_on_both_sides_of_the_small_launch(prec, shape):
+    """One field of 152 x 128 x 64 cells is the last export with a cell for each thread; two fields of it, and one of a ragged
+    grid with a few cells more, take four a thread: the values are those that were set."""
+    import torch
+    assert shape[0] * shape[1] * shape[2] - 152 * 128 * 64 in (0, 1019)
+    g = torch.Generator(device="cuda").manual_seed(4)
+    e, u = (torch.rand(shape, generator=g, dtype=torch.float64, device="cuda") + 0.5 for _ in range(2))
+    e, u = e.float().double(), u.float().double()
+    z = torch.zeros_like(e)
+    h = clv.Hydro(*shape, 0.2, 0.2, 0.2, 0.5, 0.01, 0.0, None, prec)
+    h.set_initial(e, u, z, z)
+    for names in (["eps"], ["ux"], ["eps", "ux"]):
+        f = h.get_device(names)
+        for k in names:
+            assert torch.equal(f[k].reshape(shape), e if k == "eps" else u), (names, k)
