@@ -526,7 +526,6 @@ __device__ __forceinline__ void shear_update(float inv, float un, const float pi
 
 template <typename R, int STAGE, bool VISC, bool STATS>
 __global__ void __launch_bounds__(kBlock) stage_kernel(const StageParams<R> p) {
-  release_next_kernel();
   enter_step_kernel();
   const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   long long row;

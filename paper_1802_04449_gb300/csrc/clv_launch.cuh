@@ -13,7 +13,10 @@ namespace clv {
 // as they start; the stage kernels, at most one wave of large CTAs, do not: the
 // small blocks of the next kernel would be placed on the SMs that are free then,
 // and the others stay empty (33 x 33 x 9 in FP64, 132 CTAs on 152 SMs: 141 us a
-// step instead of 84).  No effect on a plain launch.
+// step instead of 84).  Nor does the direct stage kernel (kernel = 1), whose
+// next launch runs the same code: ten steps of 33 x 33 x 9 viscous cells in FP32
+// took 282 us with a release at its start, 273 as plain launches and 240
+// without one; 45 x 45 x 21 cells 479, 494 and 424.  No effect on a plain launch.
 __device__ __forceinline__ void enter_step_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void release_next_kernel() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 template <typename... P, typename... A>
