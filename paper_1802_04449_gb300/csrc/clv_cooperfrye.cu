@@ -257,7 +257,12 @@ __global__ void cf_reduce_kernel(const double* __restrict__ partial, int nchunk,
 
 // ---- host side
 
-constexpr int kTargetCtas = 1216;   // momentum tiles x element chunks x species, about 8 per SM
+// Momentum tiles x element chunks x species, about 8 per SM.  A rule for whole
+// waves of resident CTAs was 2.3% faster on 60,000 elements x 3 x 41 x 15 x 48
+// points in FP32 (3.60 -> 3.52 ms), but 5% slower on 20,000 (1.24 -> 1.31) and on
+// 3 x 20 x 10 x 24 points (0.65 -> 0.68), and 12% in FP64 on 3 x 5 x 5 x 8 points
+// (16.8 -> 18.7), where the CTAs of an SM share its FP64 pipe.
+constexpr int kTargetCtas = 1216;
 
 struct Plan {
   long long npts, nthr;

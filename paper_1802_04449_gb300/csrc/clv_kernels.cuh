@@ -461,8 +461,8 @@ __device__ __forceinline__ void shear_source(double geo, const double u[4], doub
 // written out and none is left for the compiler to form, which it did in
 // another way in each kernel.  APART keeps what the three kernels had: bit m,
 // the product u~^m u~^m of sigma^{mm} is rounded before it is subtracted, and
-// with any bit so is u~^eta / tau.  The gathered sum of FP64 would be 1% faster
-// (20 steps of 97 x 97 x 41 cells: 3.85 ms against 3.89).
+// with any bit so is u~^eta / tau.  The gathered sum of FP64 would be 1-2% faster
+// (97 x 97 x 41 cells: stages of 66.8 and 76.5 us against 67.4 and 77.8).
 template <int APART>
 __device__ __forceinline__ void shear_source(float geo, const float u[4], float du[4][4], const float pi[10], float e,
                                              float P, float inv_taupi, const IsCoef<float>& is, float* S) {
@@ -809,7 +809,7 @@ __global__ void __launch_bounds__(kBlock) stage_kernel(const StageParams<R> p) {
 // (STATS) reduces sum T~^{tau tau} and max eps.
 // blocks of 256 threads (or as many smaller ones) per SM: the dependent table
 // lookups of the root solve need the occupancy.  In FP32 six, with 40 registers
-// and a spill of 64 to 116 bytes, are 10% faster than four (261 x 261 x 121 cells: 239 -> 213
+// and a spill of 64 to 116 bytes, are 12% faster than four (261 x 261 x 121 cells: 249 -> 219
 // us a launch); with the network, which then spills more, four are best
 template <typename R, int GUESS>
 struct RecoverMinBlocks {

@@ -252,8 +252,8 @@ __device__ __forceinline__ void stage_tile_body(const StageParams<R>& p, const E
   // Thread = cell (ta, tb) below ncell, = y-interface (ta, tb) below NHY and
   // (FP32) = eta-interface tid, in rows of TK + 1, below NHK: each list fills
   // whole warps, and the last threads, with least to do, take the staging
-  // first (8 x 41 tiles, 97 x 97 x 41: stage 1 67.8 -> 65.7 us against a thread
-  // per position).  A batch in FP32 keeps a thread per position of (TJ+1) rows of
+  // first (8 x 41 tiles, 97 x 97 x 41: stages 69.8 -> 67.4 and 80.4 -> 77.8 us
+  // against a thread per position).  A batch in FP32 keeps a thread per position of (TJ+1) rows of
   // TK + 1: in the loop over its items the other one spills 200 bytes (twelve
   // events, 40 steps: 65 -> 79 ms).
   constexpr bool POSITIONS = !F64 && BATCH;
